@@ -142,9 +142,12 @@ typedef struct np_config {
   int32_t parent_grid;   /* persistent parent CTAs; 0 = resident capacity */
   int32_t serial;        /* NP_SERIAL_*: where the children of parents below the threshold run */
   int32_t small_parents; /* grid-host form, while driver: before the while loop and at the end
-                            of each body one CTA runs whole levels itself while the frontier
-                            has at most this many parents (<= NP_SMALL_PARENTS_MAX) and at
-                            most 16384 children in all; 0 = off */
+                            of each body small levels run whole, without grids; 0 = off.
+                            BFS: in one CTA, while the frontier has at most this many parents
+                            (<= NP_SMALL_PARENTS_MAX) and at most 16384 children in all.
+                            SSSP: in one cluster of CTAs, up to 8 times this many parents; a
+                            round may leave the farther part of a slowly growing frontier to
+                            later rounds, so levels and items in np_stats count rounds */
   int32_t sweep_parents; /* level loops: levels with at least this many parents form the
                             next frontier by a sweep (see below); 0 = every level appends */
   int32_t reserved[1];   /* must be zero */

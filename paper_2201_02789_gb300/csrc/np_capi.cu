@@ -73,7 +73,7 @@ np_status solve(np_ctx* c, int kind, const np_csr* g, int src, int* level, unsig
   a.b.level = level;
   a.b.dist = dist;
   a.b.stamp = wsp<int>(c->w, c->w.lay.off_stamp);
-  if (p.sweep) a.n_vertices = g->n;
+  a.n_vertices = g->n;
   if (kind == 1) {
     NP_TRY(ensure_dtag(c, g->n));
     a.b.dtag = c->dtag;
@@ -146,7 +146,7 @@ np_status solve_multi(np_ctx* c, int kind, const np_csr* g, int nsrc, const int3
   a.b.stamp = wsp<int>(c->w, c->w.lay.off_stamp);
   a.b.vmask = (int)(ld - 1);
   // a swept frontier sweeps every query's state (padding entries stay unreached)
-  if (p.sweep) a.n_vertices = (int)total;
+  a.n_vertices = (int)total;
   if (kind == 1) {
     NP_TRY(ensure_dtag(c, total));
     a.b.dtag = c->dtag;

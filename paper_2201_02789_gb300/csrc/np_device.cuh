@@ -31,5 +31,5 @@
 // level L + 2 will use.
 #pragma once
 
-#include "np_loop.cuh"   // and, through it, every part in order:
-// np_state, np_sinks, np_bodies, np_child, np_parent, np_loop
+#include "np_small.cuh"   // and, through it, every part in order:
+// np_state, np_sinks, np_bodies, np_child, np_parent, np_loop, np_small

@@ -384,6 +384,8 @@ Plan make_plan(const BodyKernels& K, const np_config& cfg) {
     p.child = form == NP_SERIAL_PACKED ? K.child_agg_pack[cfi] : K.child_agg[cfi];
     p.loop = K.level_loop_agg[cfi];
     p.small = cfg.small_parents > 0 ? K.level_small : nullptr;
+    p.small_smem = p.small ? (size_t)K.level_small_smem : 0;
+    p.small_cluster = p.small && K.level_small_cluster ? 1 : 0;
     p.child_idle = cfg.threshold == INT32_MAX && form != NP_SERIAL_PACKED;
     if (sweeps(cfg) && K.parent_sweep) {
       p.parent = K.parent_sweep;
@@ -463,18 +465,28 @@ namespace {
 
 // A launch that may be scheduled while its predecessor on the stream is still
 // running (programmatic dependent launch); the kernel waits for it itself.
-cudaError_t launch_pdl(const void* fn, dim3 grid, dim3 block, void** args, cudaStream_t s, bool pdl) {
-  if (!pdl) return cudaLaunchKernel(fn, grid, block, args, 0, s);
+cudaError_t launch_pdl(const void* fn, dim3 grid, dim3 block, void** args, cudaStream_t s, bool pdl,
+                       size_t smem = 0, int cluster = 0) {
+  if (!pdl && !cluster) return cudaLaunchKernel(fn, grid, block, args, smem, s);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
-  cfg.dynamicSmemBytes = 0;
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchAttribute at[2];
+  unsigned n = 0;
+  if (pdl) {
+    at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[n++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (cluster) {
+    at[n].id = cudaLaunchAttributeClusterDimension;
+    at[n].val.clusterDim.x = (unsigned)cluster;
+    at[n].val.clusterDim.y = 1;
+    at[n++].val.clusterDim.z = 1;
+  }
   cfg.attrs = at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = n;
   return cudaLaunchKernelExC(&cfg, fn, args);
 }
 
@@ -651,6 +663,42 @@ np_status chunk_graph(Engine& e, Workspace& w, const Plan& p, const Args& a, con
   return cache_graph(w, key, graph, out);
 }
 
+// CTAs of the small-level loop (its cluster, or one) and threads of each; sets
+// the kernel's shared memory and cluster limits. A cluster of 16 CTAs where
+// the device can hold one, else of 8 (the portable size).
+static np_status small_shape(Engine& e, const Plan& p, int* ctas, int* threads) {
+  if (p.small_smem)
+    NP_CK(cudaFuncSetAttribute(p.small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.small_smem));
+  *ctas = 1;
+  *threads = 1024;
+  if (!p.small_cluster) return NP_OK;
+  *threads = kClThreads;
+  NP_CK(cudaFuncSetAttribute(p.small, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+  auto key = std::make_pair(p.small, -1);
+  auto it = e.occ.find(key);
+  if (it == e.occ.end()) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(kClMax);
+    cfg.blockDim = dim3(kClThreads);
+    cfg.dynamicSmemBytes = p.small_smem;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = kClMax;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, p.small, &cfg) != cudaSuccess) {
+      cudaGetLastError();
+      n = 0;
+    }
+    it = e.occ.emplace(key, n > 0 ? kClMax : 8).first;
+  }
+  *ctas = it->second;
+  return NP_OK;
+}
+
 np_status add_while_node(Engine& e, LevelState* st, cudaGraph_t graph, const cudaGraphNode_t* deps, size_t ndeps,
                          const Plan& p, const Args& a, const Grids& g, int K, cudaGraphNode_t* node) {
   cudaGraphConditionalHandle h;
@@ -658,16 +706,26 @@ np_status add_while_node(Engine& e, LevelState* st, cudaGraph_t graph, const cud
   // With the small-level loop: one run of it before the loop, which sets the
   // loop's condition itself (a traversal that stays small never enters it).
   cudaGraphNode_t pre;
+  int sctas = 1, sthreads = 1024;
   if (p.small) {
+    NP_TRY(small_shape(e, p, &sctas, &sthreads));
     Args sa = a;
     int k0 = 0, in_body = 0;
     void* sargs[] = {&sa, &h, &k0, &in_body};
     cudaKernelNodeParams kp = {};
     kp.func = const_cast<void*>(p.small);
-    kp.gridDim = dim3(1);
-    kp.blockDim = dim3(1024);
+    kp.gridDim = dim3(sctas);
+    kp.blockDim = dim3(sthreads);
+    kp.sharedMemBytes = (unsigned)p.small_smem;
     kp.kernelParams = sargs;
     NP_CK(cudaGraphAddKernelNode(&pre, graph, deps, ndeps, &kp));
+    if (p.small_cluster) {
+      cudaKernelNodeAttrValue av = {};
+      av.clusterDim.x = (unsigned)sctas;
+      av.clusterDim.y = 1;
+      av.clusterDim.z = 1;
+      NP_CK(cudaGraphKernelNodeSetAttribute(pre, cudaKernelNodeAttributeClusterDimension, &av));
+    }
     deps = &pre;
     ndeps = 1;
   }
@@ -688,7 +746,8 @@ np_status add_while_node(Engine& e, LevelState* st, cudaGraph_t graph, const cud
     Args sa = a;
     int in_body = 1;
     void* sargs[] = {&sa, &h, &K, &in_body};
-    le = launch_pdl(p.small, dim3(1), dim3(1024), sargs, e.cap_stream, kPdl);
+    le = launch_pdl(p.small, dim3(sctas), dim3(sthreads), sargs, e.cap_stream, kPdl, p.small_smem,
+                    p.small_cluster ? sctas : 0);
   } else {
     void* cargs[] = {&st, &h, &K};
     le = launch_pdl((const void*)set_cond_kernel, dim3(1), dim3(1), cargs, e.cap_stream, kPdl);

@@ -3,7 +3,13 @@
 
 namespace nestpar {
 const BodyKernels& sssp64_kernels() {
-  static const BodyKernels t = with_sweep<Sssp64SweepBody, 1>(make_table<Sssp64Body>());
+  static const BodyKernels t = [] {
+    BodyKernels k = with_sweep<Sssp64SweepBody, 1>(make_table<Sssp64Body>());
+    k.level_small = (const void*)sssp_cluster<Sssp64Body>;
+    k.level_small_smem = (int)kClusterSmem;
+    k.level_small_cluster = true;
+    return k;
+  }();
   return t;
 }
 }  // namespace nestpar

@@ -131,7 +131,8 @@ struct __align__(16) LevelState {
   int pack_records[4];
   int pack_items[4];
   int pack_ticket[4];
-  int pad2[4];
+  int small_n;                   // the cluster loop: entries written to the frontier it leaves
+  int pad2[3];
 };
 
 __device__ __forceinline__ unsigned long long level_epoch(const LevelState* st, int L) {
@@ -231,7 +232,7 @@ struct Args {
   int4* prec;
   int* pfirst;
   int small_parents;             // > 0: the while body's one-CTA loop runs levels of at most this many parents
-  int n_vertices;                // swept frontier: state elements the sweep visits
+  int n_vertices;                // elements of the vertex state (level loops): what the frontier sweep visits
   int sweep_parents;             // swept frontier: levels with at least this many parents sweep (0 = none)
   // swept frontier of a serving pool: the sweep skips the chunks of slots
   // that hold no query (slot = element >> sweep_lg, sweep_lg >= 11), or NULL

@@ -1,5 +1,7 @@
 // Instantiates every kernel of one body and fills its table.
 #pragma once
+#include <type_traits>
+
 #include "np_device.cuh"
 #include "np_kernels.h"
 
@@ -46,8 +48,8 @@ inline BodyKernels make_table() {
   t.child_agg_pack[2] = (const void*)child_agg_pack<Body, 4>;
   t.child_agg_pack[3] = (const void*)child_agg_pack<Body, 8>;
   t.child_agg_pack[4] = (const void*)child_agg_pack<Body, 16>;
-  // level loops only: bodies that append to the next frontier
-  t.level_small = Body::kPushes ? (const void*)level_small<Body> : nullptr;
+  // level loops only: BFS (the packed SSSP has a form of its own, sssp_cluster)
+  if constexpr (std::is_same_v<Body, BfsBody>) t.level_small = (const void*)level_small<Body>;
   return t;
 }
 

@@ -1,0 +1,95 @@
+"""The cluster loop over small SSSP levels (np_config.small_parents) where it can go wrong:
+the distance window, lists that run full, and the changes to and from the grids. Distances
+are whole numbers and must match the oracle bit for bit."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from gpu_util import DevGraph, sssp
+from invariants import csr_from_edges
+from paper_2201_02789_gb300 import gen
+from paper_2201_02789_gb300 import nestpar as npb
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    c = npb.Context(0)
+    yield c
+    c.close()
+
+
+def _road(rows, cols, lo, hi):
+    """A grid whose frontier grows past the window's size (and, at 330 x 310, past the frontier limit
+    if nothing is deferred)."""
+    g = gen.road_grid(rows, cols, seed=9, weights=None)
+    g.w = gen.uniform_int(9, gen.S_WEIGHT, 0, g.m, lo, hi).astype(np.uint32)
+    return g
+
+
+def _wide(hubs, degree, seed):
+    """0 -> hubs vertices of `degree` children each, all into one pool: parents of 512 children or
+    more, more of them than one CTA (64) or the cluster (1024) can publish in a round."""
+    rng = np.random.default_rng(seed)
+    pool = hubs + 1 + rng.integers(0, 4000, size=(hubs, degree))
+    src = np.concatenate([np.zeros(hubs, np.int64), np.repeat(np.arange(1, hubs + 1), degree)])
+    dst = np.concatenate([np.arange(1, hubs + 1), pool.reshape(-1)])
+    order = np.argsort(src, kind="stable")
+    n = hubs + 4001
+    row_ptr = np.zeros(n + 1, np.int32)
+    row_ptr[1:] = np.cumsum(np.bincount(src, minlength=n))
+    w = rng.integers(1, 256, size=len(src)).astype(np.uint32)
+    return gen.Csr(n, row_ptr, dst[order].astype(np.int32), w)
+
+
+def _pulse():
+    """Few vertices, then 30000, then few again: the grids take over and give back."""
+    rng = np.random.default_rng(5)
+    edges = [(0, 1), (1, 2)] + [(2, 3 + i) for i in range(30000)]
+    edges += [(3 + i, 30003 + int(rng.integers(0, 50))) for i in range(30000)]
+    edges += [(30003 + i, 30053 + i % 7) for i in range(50)] + [(30053 + i, 30060) for i in range(7)]
+    edges += [(30060 + i, 30061 + i) for i in range(20)]
+    rp, col, w = csr_from_edges(30081, edges, [int(x) for x in rng.integers(1, 256, size=len(edges))])
+    return gen.Csr(30081, rp, col, w)
+
+
+GRAPHS = {
+    "road-300": lambda: _road(300, 300, 1, 255),
+    "road-330x310": lambda: _road(330, 310, 1, 255),
+    "road-zero-weights": lambda: _road(120, 130, 0, 3),
+    "road-equal-weights": lambda: _road(200, 201, 7, 7),
+    "road-large-weights": lambda: _road(230, 220, 1, 4000000),
+    "wide-70": lambda: _wide(70, 515, 1),
+    "wide-1100": lambda: _wide(1100, 513, 2),
+    "wide-3000": lambda: _wide(3000, 520, 3),
+    "pulse": _pulse,
+    "rmat-13007": lambda: gen.rmat(14, 12, seed=21, n=13007, m=13007 * 12),
+    "rmat-17001": lambda: gen.rmat(15, 24, seed=22, n=17001, m=17001 * 24),
+}
+
+
+@pytest.mark.parametrize("name", list(GRAPHS))
+def test_distances(ctx, name):
+    g = GRAPHS[name]()
+    dg = DevGraph(g)
+    for src in (0, g.n // 2):
+        ref = oracle.sssp(g.row_ptr, g.col, g.w, src)
+        for kw in ({}, {"small_parents": 300}, {"small_parents": 5, "unroll": 1}, {"sweep_parents": 0, "unroll": 2}):
+            d, st = sssp(ctx, dg, src, npb.config("tca", **kw), stats=True)
+            np.testing.assert_array_equal(d, ref)
+            assert st["error"] == 0 and st["timeouts"] == 0
+
+
+def test_several_sources_share_the_window(ctx):
+    """Queries of one call share one window, whatever their distances."""
+    g = _road(150, 140, 1, 255)
+    dg = DevGraph(g)
+    sources = [0, g.n - 1, g.n // 2, 139, 77]
+    ld = npb.multi_stride(g.n)
+    dist = torch.empty(len(sources), ld, dtype=torch.int32, device="cuda:0")
+    npb.np_sssp_multi(ctx.handle, dg.csr, sources, dist, ld, npb.config("tca"), stats=True)
+    out = dist.cpu().numpy().view(np.uint32)
+    for q, s in enumerate(sources):
+        np.testing.assert_array_equal(out[q, :g.n], oracle.sssp(g.row_ptr, g.col, g.w, s))
