@@ -733,8 +733,12 @@ def run_ours(args, ws, rank, local):
     # the while loop) + per while-body iteration `unroll` x (parent, child[, sweep]) + the
     # condition kernel (the small-level loop); a tessellation launches init, parent and child
     # (no child when the threshold launches nothing and no children are packed for it)
+    # a tessellation with spread children launches its count and point grids
     if wl["kind"] == "bezier":
-        per_solve = 2 if cfg.threshold == npb.INT32_MAX and cfg.serial != npb.NP_SERIAL_PACKED else 3
+        if cfg.serial == npb.NP_SERIAL_SPREAD:
+            per_solve = 2
+        else:
+            per_solve = 2 if cfg.threshold == npb.INT32_MAX and cfg.serial != npb.NP_SERIAL_PACKED else 3
     elif wl["kind"] == "tc":
         per_solve = 4          # level-state reset, parent, child, partial-count sum
     else:
@@ -792,6 +796,11 @@ def run_ours(args, ws, rank, local):
     child_name = "child_agg_pack" if cfg.serial == npb.NP_SERIAL_PACKED else "child_agg"
     kernels = {child_name: (prof["child_ms"], prof["child_launches"], kb["child"]),
                ("parent_cta" if cta else "parent_warp"): (prof["parent_ms"], prof["parent_launches"], kb["parent"])}
+    if wl["kind"] == "bezier" and cfg.serial == npb.NP_SERIAL_SPREAD:
+        # count grid: control points in, one word per curve out; point grid: that word, the control
+        # points and the offset per curve, 8 B per point
+        kernels = {"bezier_count": (prof["parent_ms"], prof["parent_launches"], 28 * pst["parents"]),
+                   "bezier_points": (prof["child_ms"], prof["child_launches"], 32 * pst["parents"] + 8 * pst["items"])}
     dom = max(kernels, key=lambda k: kernels[k][0])
     k_ms, k_launches, k_bytes = kernels[dom]
     per_launch_bytes = k_bytes * prof_runs / max(k_launches, 1)
@@ -860,13 +869,14 @@ def run_ours(args, ws, rank, local):
             "warmup": args.warmup, "ms_per_step": ms_per_step, "higher_is_better": True, "scaling": "weak",
             "vs_baseline": None, "dtype": {"bezier": "f32", "tc": "i32"}.get(wl["kind"], "u32"), "data": "synthetic",
             "config": dict(wl["config"], l2=L2_NOTE),
-            "form": (("threshold INT32_MAX (no child launches: the serialised children run in the parent "
-                      "warps, a whole warp per parent of 32 or more), " if wl["kind"] == "bezier" else
+            "form": (("threshold INT32_MAX (no child launches: a count grid over the curves, then a grid over "
+                      "their points, one warp per curve), " if wl["kind"] == "bezier" else
                       "threshold INT32_MAX (no child launches: the serialised children spread over the "
                       "parent warps), ") if cfg.threshold == npb.INT32_MAX else
                      f"threshold {cfg.threshold} + coarsening {cfg.cfactor} ({cfg.child_block}-thread child blocks) "
                      "+ grid aggregation (atomic scan), ") + (
-                        "one fixed pass replayed as a CUDA graph" if wl["kind"] in ("bezier", "tc") else
+                        "one fixed pass" if wl["kind"] == "bezier" else
+                        "one fixed pass replayed as a CUDA graph" if wl["kind"] == "tc" else
                         f"persistent cooperative level loop on {cfg.parent_grid} CTAs"
                         if cfg.driver == npb.NP_DRIVER_PERSISTENT else "while-graph level loop"),
             "ms_per_solve": {"median": statistics.median(ms), "min": min(ms)},

@@ -97,7 +97,9 @@ typedef int32_t np_status;
  * grid-host aggregation under a graph, chunk or host driver, where `serial`
  * chooses:
  *   NP_SERIAL_SPREAD  in the parent kernel (32-parent warp tiles), the items
- *                     of a warp's parents spread over the warp's lanes;
+ *                     of a warp's parents spread over the warp's lanes (the
+ *                     tessellation: with the points of the other curves, in
+ *                     one grid over the output, a warp per curve);
  *   NP_SERIAL_BLOCK   in the parent kernel (CTA tiles of parent_block
  *                     parents), the items of the tile's parents spread over
  *                     the CTA: the tile's records are staged in shared memory

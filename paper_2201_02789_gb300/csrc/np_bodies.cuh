@@ -21,7 +21,6 @@ struct BfsBody {
   static constexpr bool kPushes = true;
   static constexpr bool kBalance = false;   // child blocks cost the same: static ranges
   static constexpr int kStage = 1;          // edge lists the child can stage: col
-  static constexpr bool kWarpLoop = false;
   static constexpr int kWarpParentRegs = NP_WARP_PARENT_MAXREG;
   static constexpr int kCtaParentRegs = NP_CTA_PARENT_MAXREG;
   struct P {
@@ -72,7 +71,6 @@ struct SsspBody {
   static constexpr bool kPushes = true;
   static constexpr bool kBalance = false;
   static constexpr int kStage = 2;          // col and w
-  static constexpr bool kWarpLoop = false;
   static constexpr int kWarpParentRegs = 96;   // (the stamp form spills at 80)
   static constexpr int kCtaParentRegs = NP_CTA_PARENT_MAXREG;
   struct P {
@@ -184,7 +182,6 @@ struct TcBody {
   static constexpr bool kPushes = false;
   static constexpr bool kBalance = true;    // block cost varies with the lists' lengths
   static constexpr int kStage = 0;
-  static constexpr bool kWarpLoop = false;
   static constexpr int kWarpParentRegs = NP_WARP_PARENT_MAXREG;
   static constexpr int kCtaParentRegs = NP_CTA_PARENT_MAXREG;
   struct P {
@@ -251,7 +248,6 @@ struct Sssp64Body {
   static constexpr bool kPushes = true;
   static constexpr bool kBalance = false;
   static constexpr int kStage = 2;          // col and w
-  static constexpr bool kWarpLoop = false;
   static constexpr int kWarpParentRegs = NP_WARP_PARENT_MAXREG;
   static constexpr int kCtaParentRegs = NP_CTA_PARENT_MAXREG;
   struct P {
@@ -383,10 +379,7 @@ struct BezierBody {
   static constexpr bool kPushes = false;
   static constexpr bool kBalance = false;
   static constexpr int kStage = 0;
-  // serialised curves of 32 points or more run with the whole parent warp (a
-  // point only stores: one parent at a time beats spreading several)
-  static constexpr bool kWarpLoop = true;
-  static constexpr int kWarpParentRegs = 64;   // (no spill: two 512-thread CTAs per SM)
+  static constexpr int kWarpParentRegs = 64;   // (No-CDP form: two 512-thread CTAs per SM)
   // (64 still fits two 512-thread CTAs per SM, as 48 does; 48 spills)
   static constexpr int kCtaParentRegs = 64;
   struct P {
@@ -436,6 +429,15 @@ struct BezierBody {
     const unsigned long long C = (unsigned long long)(cx * cx) + (unsigned long long)(cy * cy);
     if (C == 0) return S > 0 ? 4096 : 4;
     if (S == 0) return 4;                                   // t = 0 exactly, in FP64 too
+    // FP32 first: S, C, their quotient and two square roots, each correctly
+    // rounded, put t within a relative 2.25 * 2^-24 (and a little) of its exact
+    // value, so unless an integer lies within 2^-21 of it the ceiling is settled
+    // (one random curve in some ten thousand goes on to the exact comparison)
+    {
+      const float t = 64.0f * sqrtf(sqrtf((float)S / (float)C));
+      const float up = ceilf(t * (1.0f + 0x1p-21f));
+      if (ceilf(t * (1.0f - 0x1p-21f)) == up) return up < 4.0f ? 4 : (up > 4096.0f ? 4096 : (int)up);
+    }
     using u128 = unsigned __int128;
     const u128 A = (u128)S << 24;                          // t^4 * C
     auto q4 = [&](unsigned long long m) -> u128 { const u128 m2 = (u128)(m * m); return m2 * m2 * C; };

@@ -173,6 +173,22 @@ np_status fixed_pass(np_ctx* c, const Args& a0, const np_config& cfg, const Body
                      cudaStream_t s) {
   Plan p = make_plan(K, cfg);
   Args a = a0;
+  if (p.points) {
+    const int occ = occupancy(c->e, p.parent, kPointBlock);
+    if (!c->e.profile) return enqueue_points(p, a, cfg.parent_grid, c->e.sms, occ, s);
+    NP_CK(cudaEventRecord(c->e.ev[0], s));
+    NP_TRY(enqueue_points(p, a, cfg.parent_grid, c->e.sms, occ, s, c->e.ev[1]));
+    NP_CK(cudaEventRecord(c->e.ev[2], s));
+    NP_CK(cudaEventSynchronize(c->e.ev[2]));
+    float t01 = 0.f, t12 = 0.f;
+    NP_CK(cudaEventElapsedTime(&t01, c->e.ev[0], c->e.ev[1]));
+    NP_CK(cudaEventElapsedTime(&t12, c->e.ev[1], c->e.ev[2]));
+    c->e.prof.parent_ms += t01;
+    c->e.prof.parent_launches += 1;
+    c->e.prof.child_ms += t12;
+    c->e.prof.child_launches += 1;
+    return NP_OK;
+  }
   Grids g = grids_for(c->e, p, cfg, count);
   if (c->e.profile) {
     NP_CK(cudaEventRecord(c->e.ev[0], s));

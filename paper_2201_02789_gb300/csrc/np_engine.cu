@@ -387,6 +387,12 @@ Plan make_plan(const BodyKernels& K, const np_config& cfg) {
     p.small_smem = p.small ? (size_t)K.level_small_smem : 0;
     p.small_cluster = p.small && K.level_small_cluster ? 1 : 0;
     p.child_idle = cfg.threshold == INT32_MAX && form != NP_SERIAL_PACKED;
+    if (K.points && form == NP_SERIAL_SPREAD) {
+      p.parent = K.points_count;
+      p.child = K.points;
+      p.child_idle = false;
+      p.points = true;
+    }
     if (sweeps(cfg) && K.parent_sweep) {
       p.parent = K.parent_sweep;
       p.child = K.child_sweep[cfi];
@@ -544,6 +550,26 @@ np_status enqueue_pass(const Plan& p, Args a, const Grids& g, bool level_mode, i
     NP_CK(launch_pdl(p.child, dim3(g.cgrid), dim3(g.cthreads), cargs, s, pdl));
   }
   if (p.sweep && level_mode) NP_CK(launch_pdl(p.sweep, dim3(sweep_grid(a, g)), dim3(256), pargs, s, pdl));
+  return NP_OK;
+}
+
+// The count grid is launched after everything before it on the stream (it may
+// follow a launch that is not a kernel, and stream capture then has no
+// programmatic edge to make of it); the point grid may be scheduled early.
+np_status enqueue_points(const Plan& p, Args a, int parent_grid, int sms, int occ_count, cudaStream_t s,
+                         cudaEvent_t mid) {
+  const int tiles = (int)(((int64_t)a.count_fixed + kPointBlock - 1) / kPointBlock);
+  const int per = kPointBlock / 32 * kPointCurves;   // curves of one point CTA
+  // CTAs over the curves, whole tiles of them, and one for the totals unless the count grid takes those
+  const int tile_ctas = kPointBlock / per;
+  a.k = tiles > kPointScanTiles ? 1 : 0;
+  const int64_t groups = (int64_t)tiles * tile_ctas + (a.k ? 0 : 1);
+  int pg = parent_grid > 0 ? parent_grid : occ_count * sms;
+  if (pg > tiles) pg = tiles;
+  void* args[] = {&a};
+  NP_CK(cudaLaunchKernel(p.parent, dim3(pg), dim3(kPointBlock), args, 0, s));
+  if (mid) NP_CK(cudaEventRecord(mid, s));
+  NP_CK(launch_pdl(p.child, dim3((unsigned)groups), dim3(kPointBlock), args, s, kPdl && !mid));
   return NP_OK;
 }
 

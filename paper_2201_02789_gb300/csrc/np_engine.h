@@ -59,6 +59,9 @@ struct Plan {
   // serialised children in the parent kernel): no child grid is launched (a
   // fixed pass, or each level of a level loop)
   bool child_idle = false;
+  // tessellation, grid-host with spread children: parent counts and scans the
+  // offsets, child runs every curve's points from them (enqueue_points)
+  bool points = false;
   int mode = M_NODP;
   int gran = G_NODP;
 };
@@ -134,6 +137,14 @@ Grids grids_for(Engine& e, const Plan& p, const np_config& cfg, int64_t max_pare
 int resolve_driver(const Plan& p, const np_config& cfg);
 
 np_status enqueue_pass(const Plan& p, Args a, const Grids& g, bool level_mode, int k, cudaStream_t s);
+// The two grids of a tessellation pass (Plan::points), on s; `mid`, if not
+// NULL, is recorded between them. The resident CTAs per SM of the count grid
+// come from the caller.
+constexpr int kPointBlock = 256;    // threads of a CTA, and curves of a count tile
+constexpr int kPointCurves = 8;     // curves of a warp of the point grid
+constexpr int kPointScanTiles = 4 * kPointBlock;   // up to here a point CTA sums the tiles before it itself
+np_status enqueue_points(const Plan& p, Args a, int parent_grid, int sms, int occ_count, cudaStream_t s,
+                         cudaEvent_t mid = nullptr);
 np_status enqueue_advance(LevelState* st, int K, cudaStream_t s, bool after_launch_free = false);
 np_status profiled_pass(Engine& e, const Workspace& w, const Plan& p, Args a, const Grids& g, bool level_mode,
                         cudaStream_t s);

@@ -34,6 +34,10 @@ struct BodyKernels {
   const void* parent_sweep;
   const void* child_sweep[kNumCF];
   const void* frontier_sweep;
+  // tessellation only (else NULL): the grid-host form with its children spread,
+  // as a count grid over the curves and a grid over their points
+  const void* points_count;
+  const void* points;
 };
 
 const BodyKernels& bfs_kernels();

@@ -406,34 +406,11 @@ __device__ __forceinline__ void parent_warp_run(const Args& a, int L, int count,
       // its own list.
       if (__ballot_sync(kFull, serial) == 0u) continue;   // (uniform) no serialised children in this tile
       const typename Body::P pm = Body::parent(b, serial ? pid : 0, base, N);
-      // Bodies with kWarpLoop: a parent with at least 32 serialised children
-      // runs them with the whole warp, one parent at a time: child j on lane
-      // j % 32, coalesced, the parent's fields taken by shuffle once.
-      const int wideN = Body::kWarpLoop && serial && N >= 32 ? N : 0;
-      const int myN = serial && wideN == 0 ? N : 0;
-      if constexpr (Body::kWarpLoop) {
-        for (unsigned wm = __ballot_sync(kFull, wideN > 0); wm; wm &= wm - 1) {
-          const int src = __ffs(wm) - 1;
-          const int n = __shfl_sync(kFull, wideN, src);
-          const typename Body::P p = Body::shfl(pm, src);
-          for (int j0 = 0; j0 < n; j0 += 32) {
-            typename Body::F f[1];
-            typename Body::P pk[1] = {p};
-            bool v[1] = {j0 + lane < n};
-            int idx[1] = {j0 + lane};
-            f[0] = v[0] ? Body::fetch(b, p, idx[0]) : typename Body::F{};
-            bool pf[1];
-            int pv[1];
-            Body::template apply_batch<1>(b, pk, idx, f, v, pf, pv);
-            if constexpr (Body::kPushes) sink.template push<1>(pf, pv);
-          }
-        }
-      }
-      // The others are spread over the warp's lanes: their children are
+      // They are spread over the warp's lanes: their children are
       // numbered in parent order, item t goes to lane t % 32, which finds its
       // parent (the first lane whose inclusive count exceeds t) by a shuffle
       // search and takes the parent's fields by shuffle.
-      int incl = myN;
+      int incl = serial ? N : 0;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
         const int x = __shfl_up_sync(kFull, incl, o);
@@ -441,9 +418,8 @@ __device__ __forceinline__ void parent_warp_run(const Args& a, int L, int count,
       }
       const int total = __shfl_sync(kFull, incl, 31);
       if (total > 0) {
-        // (the tessellation's 36-byte parents take two items per lane)
-        constexpr int KS = sizeof(typename Body::P) > 16 ? 2 : NP_SPREAD_BATCH;
-        const int excl = incl - myN;
+        constexpr int KS = NP_SPREAD_BATCH;
+        const int excl = incl - (serial ? N : 0);
         for (int t0 = 0; t0 < total; t0 += 32 * KS) {
           typename Body::F f[KS];
           typename Body::P pk[KS];

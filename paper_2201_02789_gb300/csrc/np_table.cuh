@@ -20,7 +20,8 @@ template <class Body>
 inline BodyKernels make_table() {
   BodyKernels t{};
   t.parent_nodp = (const void*)parent_warp<Body, 0>;
-  t.parent_grid_host = (const void*)parent_warp<Body, 1>;
+  // (the tessellation has its count and point grids instead)
+  if constexpr (!Body::kOffsets) t.parent_grid_host = (const void*)parent_warp<Body, 1>;
   t.parent_nodp_cta = (const void*)parent_kernel<Body, G_NODP, 1>;
   fill_parent_row<Body, G_NONE>(t.parent[0]);
   fill_parent_row<Body, G_WARP>(t.parent[1]);
@@ -36,19 +37,21 @@ inline BodyKernels make_table() {
   t.child_agg[2] = (const void*)child_agg<Body, 4>;
   t.child_agg[3] = (const void*)child_agg<Body, 8>;
   t.child_agg[4] = (const void*)child_agg<Body, 16>;
-  t.level_loop_nodp = (const void*)level_loop<Body, 0, 1>;
-  t.level_loop_agg[0] = (const void*)level_loop<Body, 1, 1>;
-  t.level_loop_agg[1] = (const void*)level_loop<Body, 1, 2>;
-  t.level_loop_agg[2] = (const void*)level_loop<Body, 1, 4>;
-  t.level_loop_agg[3] = (const void*)level_loop<Body, 1, 8>;
-  t.level_loop_agg[4] = (const void*)level_loop<Body, 1, 16>;
+  if constexpr (Body::kPushes) {   // level loops: bodies that append to the next frontier
+    t.level_loop_nodp = (const void*)level_loop<Body, 0, 1>;
+    t.level_loop_agg[0] = (const void*)level_loop<Body, 1, 1>;
+    t.level_loop_agg[1] = (const void*)level_loop<Body, 1, 2>;
+    t.level_loop_agg[2] = (const void*)level_loop<Body, 1, 4>;
+    t.level_loop_agg[3] = (const void*)level_loop<Body, 1, 8>;
+    t.level_loop_agg[4] = (const void*)level_loop<Body, 1, 16>;
+  }
   t.parent_cta = (const void*)parent_cta<Body>;
   t.child_agg_pack[0] = (const void*)child_agg_pack<Body, 1>;
   t.child_agg_pack[1] = (const void*)child_agg_pack<Body, 2>;
   t.child_agg_pack[2] = (const void*)child_agg_pack<Body, 4>;
   t.child_agg_pack[3] = (const void*)child_agg_pack<Body, 8>;
   t.child_agg_pack[4] = (const void*)child_agg_pack<Body, 16>;
-  // level loops only: BFS (the packed SSSP has a form of its own, sssp_cluster)
+  // small levels: BFS (the packed SSSP has a form of its own, sssp_cluster)
   if constexpr (std::is_same_v<Body, BfsBody>) t.level_small = (const void*)level_small<Body>;
   return t;
 }

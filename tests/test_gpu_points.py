@@ -1,0 +1,87 @@
+"""The tessellation's count and point grids at the edges of their tiles (256 curves, 64 per
+point CTA, 1024 tiles summed by the point CTAs themselves), with parent subsets and a capacity
+that falls inside a tile. Offsets exact; points |g - r| <= 1e-5 max(|r|, 1) as everywhere
+(three exact integer weights times products rounded twice: below 1e-6)."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from gpu_util import bezier
+from invariants import bezier_tolerance_ok
+from paper_2201_02789_gb300 import gen
+from paper_2201_02789_gb300 import nestpar as npb
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    c = npb.Context(0)
+    yield c
+    c.close()
+
+
+def _few_points(n):
+    """n curves of 4 to 14 points (nearly straight), every 1000th a random one."""
+    ctrl = gen.bezier_curves(n, seed=51)
+    mid = (ctrl[:, 0] + ctrl[:, 2]) * np.float32(0.5)
+    flat = mid + (ctrl[:, 1] - mid) * np.float32(1e-4)
+    out = ctrl.copy()
+    out[:, 1] = flat
+    out[::1000] = ctrl[::1000]
+    return np.ascontiguousarray(out)
+
+
+@pytest.mark.parametrize("nc", [1, 8, 63, 64, 65, 255, 256, 257, 512, 4097, 262144, 262145, 300001])
+def test_tile_edges(ctx, nc):
+    ctrl = _few_points(nc) if nc > 10000 else gen.bezier_curves(nc, seed=52)
+    ref_off, ref_pts = oracle.bezier(ctrl)
+    for kw in ({}, {"threshold": npb.INT32_MAX, "parent_grid": 3}):
+        status, off, pts, st = bezier(ctx, ctrl, npb.config("tca", **kw), cap=int(ref_off[-1]))
+        assert status == npb.NP_OK and st["error"] == 0
+        np.testing.assert_array_equal(off, ref_off)
+        ok, worst = bezier_tolerance_ok(pts, ref_pts)
+        assert ok, worst
+        assert st["items"] == ref_off[-1] and st["parents"] == nc
+        big = int((np.diff(ref_off) >= 32).sum()) if not kw else 0
+        assert st["launch_parents"] == big and st["serial_parents"] == nc - big
+
+
+@pytest.mark.parametrize("nc", [700, 262500])
+def test_capacity_inside_a_tile(ctx, nc):
+    ctrl = _few_points(nc)
+    ref_off, ref_pts = oracle.bezier(ctrl)
+    fit = nc - 300                       # the last curve that fits, in the middle of a tile
+    cap = int(ref_off[fit + 1]) + 1
+    status, off, pts, st = bezier(ctx, ctrl, npb.config("tca"), cap=cap, check=False)
+    assert status == npb.NP_ERR_CAPACITY
+    np.testing.assert_array_equal(off, ref_off)
+    inside = int(np.searchsorted(ref_off, cap, side="right") - 1)
+    ok, worst = bezier_tolerance_ok(pts[:ref_off[inside]], ref_pts[:ref_off[inside]])
+    assert ok, worst
+    assert np.isnan(pts[ref_off[inside]:cap]).all()      # a curve that does not fit writes nothing
+    assert st["items"] == ref_off[inside]
+
+
+def test_parent_subset_with_padding(ctx):
+    ctrl = gen.bezier_curves(600, seed=53)
+    ids = np.arange(599, -1, -1, dtype=np.int32)[:520].copy()
+    ids[[0, 255, 256, 300, 519]] = -1
+    counts = np.array([oracle.bezier_count(ctrl[i]) if i >= 0 else 0 for i in ids])
+    dev = "cuda:0"
+    c_d, id_d = torch.from_numpy(ctrl).to(dev), torch.from_numpy(ids).to(dev)
+    off = torch.full((len(ids) + 1,), -7, dtype=torch.int32, device=dev)
+    pts = torch.empty((int(counts.sum()), 2), dtype=torch.float32, device=dev)
+    body = npb.np_body(kind=npb.NP_BODY_BEZIER_EVAL, ctrl=c_d.data_ptr(), offsets=off.data_ptr(),
+                       points=pts.data_ptr(), cap=int(counts.sum()))
+    _, st = npb.np_run_nested(ctx.handle, npb.np_parents(id_d.data_ptr(), len(ids)), npb.NP_COUNT_BEZIER, None, body,
+                              npb.config("tca"), stats=True)
+    o, p = off.cpu().numpy(), pts.cpu().numpy()
+    first = np.concatenate([[0], np.cumsum(counts)])
+    assert st["parents"] == (ids >= 0).sum() and o[-1] == first[-1]
+    np.testing.assert_array_equal(o[:-1][ids >= 0], first[:-1][ids >= 0])
+    assert (o[:-1][ids < 0] == -7).all()                 # padding holds no parent: its offset is not written
+    for k in np.flatnonzero(ids >= 0)[::7]:
+        for j in (0, counts[k] - 1):
+            assert bezier_tolerance_ok(p[first[k] + j], oracle.bezier_point(ctrl[ids[k]], counts[k], j))[0]
