@@ -189,6 +189,7 @@ np_status fixed_pass(np_ctx* c, const Args& a0, const np_config& cfg, const Body
     c->e.prof.child_launches += 1;
     return NP_OK;
   }
+  NP_TRY(plan_map(K, cfg, a.n_vertices, &p));
   Grids g = grids_for(c->e, p, cfg, count);
   if (c->e.profile) {
     NP_CK(cudaEventRecord(c->e.ev[0], s));
@@ -392,6 +393,7 @@ np_status np_triangles(np_ctx* c, const np_csr* dag, uint64_t* count, const np_c
   a.row_ptr = dag->row_ptr;
   a.b.col = dag->col_idx;
   a.b.row_ptr = dag->row_ptr;
+  a.n_vertices = dag->n;
   a.b.acc = c->tri;
   NP_TRY(fixed_pass(c, a, *cfg, tc_kernels(), dag->n, s));
   sum_u64_kernel<<<1, 256, 0, s>>>(c->tri, kTcSlots, reinterpret_cast<unsigned long long*>(count), 0);
@@ -500,6 +502,7 @@ np_status np_run_nested(np_ctx* c, const np_parents* parents, int32_t count_kind
     a.b.stamp = body->stamp;
   } else if (body->kind == NP_BODY_TRIANGLES) {
     a.L_fixed = 0;
+    a.n_vertices = g->n;
     a.b.row_ptr = g->row_ptr;
     a.b.acc = reinterpret_cast<unsigned long long*>(body->tri_counts);
   } else {

@@ -317,12 +317,12 @@ np_status ws_ensure(Workspace& w, int64_t parents) {
   return NP_OK;
 }
 
-int occupancy(Engine& e, const void* fn, int block) {
-  auto key = std::make_pair(fn, block);
+int occupancy(Engine& e, const void* fn, int block, size_t smem) {
+  auto key = std::make_pair(fn, block + (int)(smem / 128) * 2048);   // (block <= 1024)
   auto it = e.occ.find(key);
   if (it != e.occ.end()) return it->second;
   int n = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, block, 0) != cudaSuccess || n < 1) n = 1;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, block, smem) != cudaSuccess || n < 1) n = 1;
   e.occ[key] = n;
   return n;
 }
@@ -415,6 +415,20 @@ Plan make_plan(const BodyKernels& K, const np_config& cfg) {
   return p;
 }
 
+np_status plan_map(const BodyKernels& K, const np_config& cfg, int n, Plan* p) {
+  if (!K.map_child || p->mode != M_GRID_HOST || p->child_idle || serial_form(cfg) == NP_SERIAL_PACKED ||
+      n > K.map_vertices)
+    return NP_OK;
+  p->child = K.map_child;
+  p->child_smem = ((size_t)n + 1023) / 1024 * 128;
+  // CTAs as small as the bitmaps leave about 50 warps to an SM: 13 of 4 warps at
+  // 16 KB, 6 of 8 at 32 KB, 3 of 16 at 64 KB, then one or two of 32
+  p->child_threads = 128;
+  while (p->child_threads < 1024 && p->child_smem > (size_t)p->child_threads * 128) p->child_threads *= 2;
+  NP_CK(cudaFuncSetAttribute(p->child, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p->child_smem));
+  return NP_OK;
+}
+
 void base_args(const Workspace& w, const np_config& cfg, Args& a) {
   std::memset(&a, 0, sizeof(a));
   a.st = w.st;
@@ -457,8 +471,8 @@ Grids grids_for(Engine& e, const Plan& p, const np_config& cfg, int64_t max_pare
   if (pg > tiles) pg = tiles;
   g.pgrid = (int)pg;
   // the persistent child grid hosts cb-thread child blocks in CTAs of at least 256 threads
-  g.cthreads = g.cblock < 256 ? 256 : g.cblock;
-  g.cgrid = p.child ? occupancy(e, p.child, g.cthreads) * e.sms : 0;
+  g.cthreads = p.child_threads ? p.child_threads : g.cblock < 256 ? 256 : g.cblock;
+  g.cgrid = p.child ? occupancy(e, p.child, g.cthreads, p.child_smem) * e.sms : 0;
   return g;
 }
 
@@ -498,7 +512,7 @@ cudaError_t launch_pdl(const void* fn, dim3 grid, dim3 block, void** args, cudaS
 
 constexpr bool kPdl = NP_PDL != 0;
 
-AggSeg make_seg(const Args& a, const Grids& g, bool level_mode) {
+AggSeg make_seg(const Plan& p, const Args& a, const Grids& g, bool level_mode) {
   AggSeg seg{};
   seg.rec = a.rec;
   seg.boff = a.boff;
@@ -510,6 +524,8 @@ AggSeg make_seg(const Args& a, const Grids& g, bool level_mode) {
   seg.cb = g.cblock;
   seg.pack = a.pack;
   seg.sweep_parents = a.sweep_parents;
+  seg.cf = a.cfactor;
+  seg.words = (int)(p.child_smem / sizeof(unsigned));
   seg.prec = a.prec;
   seg.pfirst = a.pfirst;
   return seg;
@@ -544,10 +560,10 @@ np_status enqueue_pass(const Plan& p, Args a, const Grids& g, bool level_mode, i
   void* pargs[] = {&a};
   NP_CK(launch_pdl(p.parent, dim3(g.pgrid), dim3(g.pblock), pargs, s, pdl));
   if (p.mode == M_GRID_HOST && !p.child_idle) {
-    AggSeg seg = make_seg(a, g, level_mode);
+    AggSeg seg = make_seg(p, a, g, level_mode);
     BodyArgs b = child_body(a, level_mode);
     void* cargs[] = {&b, &seg};
-    NP_CK(launch_pdl(p.child, dim3(g.cgrid), dim3(g.cthreads), cargs, s, pdl));
+    NP_CK(launch_pdl(p.child, dim3(g.cgrid), dim3(g.cthreads), cargs, s, pdl, p.child_smem));
   }
   if (p.sweep && level_mode) NP_CK(launch_pdl(p.sweep, dim3(sweep_grid(a, g)), dim3(256), pargs, s, pdl));
   return NP_OK;
@@ -591,10 +607,10 @@ np_status profiled_pass(Engine& e, const Workspace& w, const Plan& p, Args a, co
   NP_CK(cudaEventRecord(e.ev[1], s));
   bool child = false, other = false;
   if (p.mode == M_GRID_HOST && !p.child_idle) {
-    AggSeg seg = make_seg(a, g, level_mode);
+    AggSeg seg = make_seg(p, a, g, level_mode);
     BodyArgs b = child_body(a, level_mode);
     void* cargs[] = {&b, &seg};
-    NP_CK(cudaLaunchKernel(p.child, dim3(g.cgrid), dim3(g.cthreads), cargs, 0, s));
+    NP_CK(cudaLaunchKernel(p.child, dim3(g.cgrid), dim3(g.cthreads), cargs, p.child_smem, s));
     child = true;
   }
   NP_CK(cudaEventRecord(e.ev[2], s));

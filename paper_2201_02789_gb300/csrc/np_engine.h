@@ -62,6 +62,9 @@ struct Plan {
   // tessellation, grid-host with spread children: parent counts and scans the
   // offsets, child runs every curve's points from them (enqueue_points)
   bool points = false;
+  // the child grid's CTA size and dynamic shared memory where the kernel has its own (0 = by child block, none)
+  int child_threads = 0;
+  size_t child_smem = 0;
   int mode = M_NODP;
   int gran = G_NODP;
 };
@@ -115,7 +118,7 @@ T* wsp(const Workspace& w, size_t off) {
   return reinterpret_cast<T*>(w.ws + off);
 }
 
-int occupancy(Engine& e, const void* fn, int block);
+int occupancy(Engine& e, const void* fn, int block, size_t smem = 0);
 np_status check_config(const np_config* cfg);
 // Where the children below the threshold run under cfg (NP_SERIAL_*): the
 // configured place for grid-host aggregation (PACKED needs threshold <= 1024,
@@ -130,6 +133,10 @@ np_config serial_for(const np_config& cfg, int64_t copies, int64_t m);
 // entry points run the appended frontier).
 bool sweeps(const np_config& cfg);
 Plan make_plan(const BodyKernels& K, const np_config& cfg);
+// Triangle counting on a graph of n vertices: the child grid with adjacency
+// bitmaps, where the plan has a child grid of whole aggregated blocks and the
+// bitmap fits.
+np_status plan_map(const BodyKernels& K, const np_config& cfg, int n, Plan* p);
 // Args of one level loop / pass over workspace `w` (vmask all ones).
 void base_args(const Workspace& w, const np_config& cfg, Args& a);
 Grids grids_for(Engine& e, const Plan& p, const np_config& cfg, int64_t max_parents);

@@ -34,6 +34,8 @@ struct BodyKernels {
   const void* parent_sweep;
   const void* child_sweep[kNumCF];
   const void* frontier_sweep;
+  const void* map_child;                      // triangle counting only (else NULL): the grid-host child grid with
+  int map_vertices;                           // adjacency bitmaps, and the most vertices it takes
   // tessellation only (else NULL): the grid-host form with its children spread,
   // as a count grid over the curves and a grid over their points
   const void* points_count;

@@ -26,7 +26,7 @@ __device__ __forceinline__ void launch_direct(const BodyArgs& b, int pid, int ba
 template <class Body, int CF>
 __device__ __forceinline__ void launch_aggregated(const BodyArgs& b, const int4* rec, const int* boff, int nrec,
                                                   int total, int child_block, unsigned* s_stat, CtaSink& sink) {
-  AggSeg s{rec, boff, nullptr, nullptr, nrec, total, 0, 0, 0, child_block, 0, nullptr, nullptr, 0, 0};   // a fixed segment
+  AggSeg s{rec, boff, nullptr, nullptr, nrec, total, 0, 0, 0, child_block, 0, nullptr, nullptr, 0, 0, 0};   // a fixed segment
   child_agg<Body, CF><<<total, child_block, 0, cudaStreamFireAndForget>>>(b, s);
   if (cudaGetLastError() != cudaSuccess) {
     // run the aggregated grid's work in this thread: parent by parent, serially

@@ -255,7 +255,8 @@ struct AggSeg {
   const int4* prec;
   const int* pfirst;
   int sweep_parents;             // level mode: levels with at least this many parents sweep (0 = none)
-  int pad;
+  int cf;                        // triangle counting: coarsening factor, and words of the CTA's adjacency bitmap
+  int words;
 };
 
 // ---------------------------------------------------------------- primitives
