@@ -146,7 +146,8 @@ typedef struct np_config {
   int32_t small_parents; /* grid-host form, while driver: before the while loop and at the end
                             of each body small levels run whole, without grids; 0 = off.
                             BFS: in one CTA, while the frontier has at most this many parents
-                            (<= NP_SMALL_PARENTS_MAX) and at most 16384 children in all.
+                            (<= NP_SMALL_PARENTS_MAX; four times as many from the start of a
+                            traversal of at most 2^20 vertices) and at most 16384 children.
                             SSSP: in one cluster of CTAs, up to 8 times this many parents; a
                             round may leave the farther part of a slowly growing frontier to
                             later rounds, so levels and items in np_stats count rounds */

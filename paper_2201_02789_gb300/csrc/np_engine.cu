@@ -386,6 +386,7 @@ Plan make_plan(const BodyKernels& K, const np_config& cfg) {
     p.small = cfg.small_parents > 0 ? K.level_small : nullptr;
     p.small_smem = p.small ? (size_t)K.level_small_smem : 0;
     p.small_cluster = p.small && K.level_small_cluster ? 1 : 0;
+    p.first = p.small ? K.first_levels : nullptr;
     p.child_idle = cfg.threshold == INT32_MAX && form != NP_SERIAL_PACKED;
     if (K.points && form == NP_SERIAL_SPREAD) {
       p.parent = K.points_count;
@@ -760,8 +761,16 @@ np_status add_while_node(Engine& e, LevelState* st, cudaGraph_t graph, const cud
     kp.blockDim = dim3(sthreads);
     kp.sharedMemBytes = (unsigned)p.small_smem;
     kp.kernelParams = sargs;
+    const bool first = p.first && a.b.vmask == INT_MAX && a.n_vertices > 0 && a.n_vertices <= kBitsMaxVertices;
+    if (first) {
+      kp.func = const_cast<void*>(p.first);
+      kp.gridDim = dim3(1);
+      kp.blockDim = dim3(1024);
+      kp.sharedMemBytes = (unsigned)bits_smem(a.n_vertices);
+      NP_CK(cudaFuncSetAttribute(p.first, cudaFuncAttributeMaxDynamicSharedMemorySize, kBitsSmem));
+    }
     NP_CK(cudaGraphAddKernelNode(&pre, graph, deps, ndeps, &kp));
-    if (p.small_cluster) {
+    if (p.small_cluster && !first) {
       cudaKernelNodeAttrValue av = {};
       av.clusterDim.x = (unsigned)sctas;
       av.clusterDim.y = 1;

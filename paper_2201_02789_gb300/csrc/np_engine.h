@@ -54,6 +54,7 @@ struct Plan {
   const void* small = nullptr;  // one-CTA small-level loop before the while loop and at each body's end (grid-host)
   size_t small_smem = 0;        // its dynamic shared memory
   int small_cluster = 0;        // and whether it runs as one cluster (1) instead of one CTA (0)
+  const void* first = nullptr;  // the loop over the first small levels in its place (one traversal, at most kBitsMaxVertices)
   const void* sweep = nullptr;  // swept frontier: the kernel that rebuilds the next frontier after each level
   // grid-host form that can give its child grid no work (threshold INT32_MAX,
   // serialised children in the parent kernel): no child grid is launched (a

@@ -29,6 +29,7 @@ struct BodyKernels {
   const void* level_small;                    // level_small<Body>: one-CTA loop over small levels (or NULL)
   int level_small_smem;                       // its dynamic shared memory
   bool level_small_cluster;                   // and whether it runs as one cluster instead of one CTA
+  const void* first_levels;                   // bfs_first_levels<Body> (or NULL): the loop before the while loop
   // swept frontier (BFS and packed SSSP only, else NULL): the grid-host parent and
   // child grids of the reducing body, and the sweep that rebuilds the frontier
   const void* parent_sweep;

@@ -1,4 +1,5 @@
-// Cluster loop over small SSSP levels, with a distance window.
+// The loops that run small levels whole: SSSP in a cluster, with a distance
+// window; BFS from its start in one CTA, with its visited set in shared memory.
 #pragma once
 #include "np_loop.cuh"
 
@@ -631,6 +632,173 @@ __global__ void __launch_bounds__(kClThreads) sssp_cluster(Args a, cudaGraphCond
       }
     }
     cudaGraphSetConditional(h, more ? 1u : 0u);
+  }
+}
+
+// -------------------------------------------------- first levels of a BFS
+//
+// One CTA runs the levels from the start of a traversal for as long as they are
+// small, with one bit per vertex in shared memory as the visited set: nothing
+// has been reached yet, so it starts empty, and a claim is a shared-memory
+// operation instead of a compare-and-swap in L2. The thread that claims a vertex
+// stores its level, loads its row bounds and queues it with its place among the
+// next level's items (one packed atomic per warp: vertices, vertices with
+// children, children), so a level needs no scan and one barrier. What is left of
+// its chain are two round trips to L2 (edges, row bounds) instead of three, and
+// what bounds a larger level is the CTA's instruction issue, not the rate of one
+// SM's L2 atomics: 8.3 us a level of 2600 children with the claims in L2, 3.7 here
+// (road grid 514 x 514, 602 levels, 5.0 -> 2.2 ms; a 4096-vertex web-like graph of
+// 18 levels 90 -> 48 us). A level of 16384 children takes about 6 us, what the
+// grids need for one however small; of 32768, 10 (R-MAT 18 then lost 14%).
+// When a level has too many parents or children the grids take over from the
+// frontier in global memory, and the body-end loop (level_small) is the one that
+// runs small levels after that.
+constexpr int kBitsQueue = 8192;        // queued parents at most (two queues of {first item, row start})
+constexpr int kBitsItems = 16384;       // children of a level (they bound its vertices, counted in 16 bits)
+constexpr int kBitsSmem = 216 * 1024;
+constexpr int kBitsMaxVertices = 1 << 20;   // 128 KB of bits; at least 5600 queued parents
+
+// Dynamic shared memory for n vertices, and the queue's size in it.
+__host__ __device__ inline int bits_words(int n) { return (n + 127) / 128 * 4; }
+__host__ __device__ inline int bits_queue(int n) {
+  const int q = (kBitsSmem - bits_words(n) * 4) / 16;
+  return q < kBitsQueue ? q : kBitsQueue;
+}
+inline size_t bits_smem(int n) { return (size_t)bits_words(n) * 4 + (size_t)bits_queue(n) * 16; }
+
+__device__ __forceinline__ int warp_segment2(const int2* seg, int n, int t) {
+  const int lane = threadIdx.x & 31;
+  int lo = 0, hi = n;
+  while (hi - lo > 32) {
+    const int stride = (hi - lo + 31) >> 5, i = lo + lane * stride;
+    const bool p = i < hi && seg[i].x <= t;
+    lo += (__popc(__ballot_sync(kFull, p)) - 1) * stride;
+    hi = min(hi, lo + stride);
+  }
+  const int i = lo + lane;
+  const bool p = i < hi && seg[i].x <= t;
+  const int r = lo + __popc(__ballot_sync(kFull, p)) - 1, j = r + 1 + lane;
+  const int at = j < n ? seg[j].x - t : 32;
+  return r + __popc(__reduce_or_sync(kFull, at < 32 ? 1u << at : 0u) & (0xffffffffu >> (31 - lane)));
+}
+
+template <class Body>
+__global__ void __launch_bounds__(1024) bfs_first_levels(Args a, cudaGraphConditionalHandle h, int, int) {
+  NP_PDL_ENTRY();
+  constexpr int KS = 4;
+  extern __shared__ __align__(16) unsigned s_bits[];
+  const int words = bits_words(a.n_vertices), cap = bits_queue(a.n_vertices);
+  int2* s_queue = reinterpret_cast<int2*>(s_bits + words);   // [2][cap]
+  // of level L at L % 3: vertices << 48 | those with children << 32 | their children
+  __shared__ unsigned long long s_tot[3];
+  LevelState* st = a.st;
+  const int tid = (int)threadIdx.x, lane = tid & 31;
+  const int limit = min(a.small_parents, kSmallParentsMax) * 4;
+  const int max_levels = __ldcg(&st->max_levels);
+  const int count0 = __ldcg(&st->count[0]);
+  const bool ran = count0 > 0 && count0 <= limit && max_levels > 0;
+  for (int i = tid; i < words / 4; i += 1024) reinterpret_cast<uint4*>(s_bits)[i] = make_uint4(0u, 0u, 0u, 0u);
+  if (tid < 3) s_tot[tid] = 0ull;
+  __syncthreads();
+  // queues the vertices id[k] with take[k] for level `to`: their row bounds, all
+  // loaded before any is used, and one atomic per warp
+  auto push = [&](auto& take, auto& id, int to, int* next) {
+    constexpr int M = sizeof(take) / sizeof(take[0]);
+    int base[M], N[M];
+    unsigned long long mine = 0ull;   // vertices << 48 | with children << 32 | children, of this thread
+#pragma unroll
+    for (int k = 0; k < M; k++) {
+      base[k] = 0;
+      N[k] = 0;
+      if (take[k]) Body::count(a, id[k], base[k], N[k]);
+    }
+#pragma unroll
+    for (int k = 0; k < M; k++)
+      mine += (take[k] ? 1ull << 48 : 0ull) + (N[k] > 0 ? 1ull << 32 : 0ull) + (unsigned)N[k];
+    if (!__any_sync(kFull, mine != 0ull)) return;
+    unsigned long long inc = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned long long x = __shfl_up_sync(kFull, inc, o);
+      if (lane >= o) inc += x;
+    }
+    unsigned long long at = 0ull;
+    if (lane == 31) at = atomicAdd(&s_tot[to % 3], inc);
+    at = __shfl_sync(kFull, at, 31) + inc - mine;
+    int pos = (int)(at >> 48), j = (int)(at >> 32 & 0xffffull);
+    unsigned first = (unsigned)at;
+#pragma unroll
+    for (int k = 0; k < M; k++) {
+      if (take[k] && next) next[pos++] = id[k];
+      if (N[k] > 0) {
+        if (j < cap) s_queue[(to & 1) * cap + j] = make_int2((int)first, base[k]);
+        j++;
+        first += (unsigned)N[k];
+      }
+    }
+  };
+  int L = 0, count = count0;
+  unsigned long long n_par = 0, n_items = 0, n_serial = 0;
+  if (ran) {
+    for (int i0 = 0; i0 < count0; i0 += 1024) {   // (the frontier itself is in global memory already)
+      const int i = i0 + tid;
+      int id[1] = {i < count0 ? __ldcg(&a.fr0[i]) : -1};
+      bool take[1] = {id[0] >= 0};
+      if (take[0]) atomicOr(&s_bits[id[0] >> 5], 1u << (id[0] & 31));
+      push(take, id, 0, nullptr);
+    }
+    __syncthreads();
+    for (;;) {
+      const unsigned long long tot = s_tot[L % 3];
+      const int segs = (int)(tot >> 32 & 0xffffull);
+      const unsigned items = (unsigned)tot;
+      count = (int)(tot >> 48);
+      // nothing left, or the grids' (a queue that overflowed has more than cap entries)
+      if (count == 0 || count > limit || segs > cap || items > (unsigned)kBitsItems || L >= max_levels) break;
+      if (tid == 0) s_tot[(L + 2) % 3] = 0ull;   // (read in level L - 1, added to from level L + 1 on)
+      n_par += (unsigned)count;
+      n_items += items;
+      n_serial += (unsigned)segs;
+      int* next = (L & 1) ? a.fr0 : a.fr1;
+      const int2* queue = s_queue + (L & 1) * cap;
+      for (int t0 = tid & ~31; t0 < (int)items; t0 += KS * 1024) {   // (uniform over the warp)
+        int v[KS];
+#pragma unroll
+        for (int k = 0; k < KS; k++) {
+          const int t = t0 + k * 1024 + lane;
+          v[k] = -1;
+          if (t - lane < (int)items) {   // (uniform)
+            // (a single traversal: an entry carries no query part)
+            const int2 q = queue[warp_segment2(queue, segs, t - lane)];
+            if (t < (int)items) v[k] = __ldg(&a.b.col[q.y + t - q.x]);
+          }
+        }
+        bool take[KS];
+#pragma unroll
+        for (int k = 0; k < KS; k++) {
+          const unsigned bit = 1u << (v[k] & 31);
+          take[k] = v[k] >= 0 && !(s_bits[v[k] >> 5] & bit) && !(atomicOr(&s_bits[v[k] >> 5], bit) & bit);
+          if (take[k]) a.b.level[v[k]] = L + 1;
+        }
+        push(take, v, L + 1, next);
+      }
+      __syncthreads();
+      L++;
+    }
+  }
+  if (tid == 0) {
+    if (ran) {
+      st->count[L % 3] = count;
+      st->count[(L + 1) % 3] = 0;
+      st->count[(L + 2) % 3] = 0;
+      add_stat(st, S_LEVELS, (unsigned long long)L);
+      add_stat(st, S_PUSHES, n_par - (L > 0 ? (unsigned long long)count0 : 0ull));
+      add_stat(st, S_PARENTS, n_par);
+      add_stat(st, S_ITEMS, n_items);
+      add_stat(st, S_SERIAL, n_serial);
+    }
+    st->base = L;
+    cudaGraphSetConditional(h, count > 0 && L < max_levels ? 1u : 0u);
   }
 }
 

@@ -1,12 +1,12 @@
-"""The cluster loop over small SSSP levels (np_config.small_parents) where it can go wrong:
-the distance window, lists that run full, and the changes to and from the grids. Distances
-are whole numbers and must match the oracle bit for bit."""
+"""The loops over small levels (np_config.small_parents) where they can go wrong: for SSSP
+the distance window, lists that run full, and the changes to and from the grids; for BFS
+the queue and its limits. Levels and distances must match the oracle bit for bit."""
 import numpy as np
 import pytest
 import torch
 
 import oracle
-from gpu_util import DevGraph, sssp
+from gpu_util import DevGraph, bfs, sssp
 from invariants import csr_from_edges
 from paper_2201_02789_gb300 import gen
 from paper_2201_02789_gb300 import nestpar as npb
@@ -93,3 +93,57 @@ def test_several_sources_share_the_window(ctx):
     out = dist.cpu().numpy().view(np.uint32)
     for q, s in enumerate(sources):
         np.testing.assert_array_equal(out[q, :g.n], oracle.sssp(g.row_ptr, g.col, g.w, s))
+
+
+# ---- BFS from its start in one CTA (visited bits in shared memory)
+
+def _fan(n, widths, seed):
+    """Levels of the given widths, every vertex of one with edges into the next (some with none,
+    some twice to the same vertex); the rest of the n vertices unreached."""
+    rng = np.random.default_rng(seed)
+    ids = rng.permutation(n)[:1 + sum(widths)]
+    src, dst, at = [ids[:0]], [ids[:0]], 1
+    prev = ids[:1]
+    for w in widths:
+        cur = ids[at:at + w]
+        at += w
+        src += [prev[rng.integers(0, max(1, len(prev) * 3 // 4), w)], prev[:1], prev[:1]]
+        dst += [cur, cur[:1], cur[:1]]
+        prev = cur
+    src, dst = np.concatenate(src), np.concatenate(dst)
+    order = np.argsort(src, kind="stable")
+    row_ptr = np.zeros(n + 1, np.int32)
+    row_ptr[1:] = np.cumsum(np.bincount(src, minlength=n))
+    return gen.Csr(n, row_ptr, dst[order].astype(np.int32)), int(ids[0])
+
+
+FANS = {
+    "words": (129, [3, 40, 80]),
+    "parents-8192": (40000, [3, 8192, 8193, 40, 8000, 5]),
+    "children-16384": (60000, [16384, 100, 16385, 7]),
+    "queue": (1 << 20, [4, 5500, 8000, 12000, 20, 7000, 9]),      # 128 KB of bits: 5632 queued parents
+    "no-bits": ((1 << 20) + 1, [4, 5500, 8000, 12000, 20, 7000, 9]),
+    "isolated": (7, []),
+}
+
+
+@pytest.mark.parametrize("name", list(FANS))
+def test_bfs_first_levels(ctx, name):
+    n, widths = FANS[name]
+    g, src = _fan(n, widths, len(name))
+    dg = DevGraph(g)
+    ref = oracle.bfs(g.row_ptr, g.col, src)
+    for kw in ({}, {"small_parents": 100}, {"sweep_parents": 0, "unroll": 1}):
+        lv, st = bfs(ctx, dg, src, npb.config("tca", **kw), stats=True)
+        np.testing.assert_array_equal(lv, ref)
+        assert st["error"] == 0 and st["parents"] == (ref >= 0).sum()
+        assert st["levels"] == ref.max() + 1 and st["pushes"] == (ref > 0).sum()
+        assert st["items"] == np.diff(g.row_ptr)[ref >= 0].sum()
+
+
+@pytest.mark.parametrize("rows,cols", [(40, 41), (300, 310)])
+def test_bfs_road(ctx, rows, cols):
+    g = gen.road_grid(rows, cols, seed=4, weights=None)
+    dg = DevGraph(g)
+    for src in (0, g.n // 2):
+        np.testing.assert_array_equal(bfs(ctx, dg, src, npb.config("tca")), oracle.bfs(g.row_ptr, g.col, src))
