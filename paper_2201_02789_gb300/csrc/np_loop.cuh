@@ -73,7 +73,7 @@ __global__ void __launch_bounds__(1024) level_loop(Args a, int max_levels) {
     const int count = __ldcg(&st->count[L % 3]);
     if (count <= 0) break;   // uniform: every CTA reads it after the same barrier
     if (blockIdx.x == 0 && threadIdx.x == 0) level_open(st, L, count);
-    parent_warp_run<Body, FORM>(a, L, count, false, s_stage, &s_stage_n, &s_stage_base);
+    parent_warp_run<Body, FORM, 0>(a, L, count, false, s_stage, &s_stage_n, &s_stage_base);
     if constexpr (FORM == 1) {
       if (!grid_barrier(st, &s_ok)) break;
       BodyArgs b = a.b;
