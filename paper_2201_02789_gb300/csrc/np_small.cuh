@@ -104,7 +104,9 @@ __device__ __forceinline__ int warp_segment(const int4* seg, int n, int t) {
 //     every CTA before the barrier, and every CTA takes the same decisions
 //     from the same headers;
 //   - a parent with kWideItems children or more is published instead of
-//     expanded, and all CTAs take a slice of it in the next round.
+//     expanded, and all CTAs take a slice of it in the next round (a round more
+//     for its children: at 512 an R-MAT graph of 3000 vertices takes 93 us
+//     instead of 82, whose hubs all have so many).
 // The window steers itself by the size of the rounds, not by the weights: no
 // cut until a slowly growing round (by less than twofold: an R-MAT frontier
 // grows tenfold and ends in a few levels, where deferring only adds rounds) has
@@ -131,7 +133,7 @@ constexpr int kClWide = 2;                      // slices of wide parents
 constexpr int kClEntries = kClPull + kClFar + kClWide;
 constexpr int kFarList = kClFar * kClThreads;
 constexpr int kWideList = 64;                   // wide parents of one CTA (16 of them: kClWide * kClThreads slices)
-constexpr int kWideItems = 512;
+constexpr int kWideItems = 2048;
 // Children of one CTA in a round beyond which it defers the rest, and of all
 // published parents together, beyond which the grids take over; first for a graph with no more vertices than the
 // frontier limit (it cannot outgrow the cluster, and the grids' fixed cost per

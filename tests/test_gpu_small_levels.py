@@ -30,8 +30,8 @@ def _road(rows, cols, lo, hi):
 
 
 def _wide(hubs, degree, seed):
-    """0 -> hubs vertices of `degree` children each, all into one pool: parents of 512 children or
-    more, more of them than one CTA (64) or the cluster (1024) can publish in a round."""
+    """0 -> hubs vertices of `degree` children each, all into one pool: wide parents (2048 children or
+    more), more of them than one CTA (64) or the cluster (1024) can publish in a round, or none."""
     rng = np.random.default_rng(seed)
     pool = hubs + 1 + rng.integers(0, 4000, size=(hubs, degree))
     src = np.concatenate([np.zeros(hubs, np.int64), np.repeat(np.arange(1, hubs + 1), degree)])
@@ -64,6 +64,9 @@ GRAPHS = {
     "wide-70": lambda: _wide(70, 515, 1),
     "wide-1100": lambda: _wide(1100, 513, 2),
     "wide-3000": lambda: _wide(3000, 520, 3),
+    "wide-70x2047": lambda: _wide(70, 2047, 4),
+    "wide-70x2048": lambda: _wide(70, 2048, 5),
+    "wide-1100x2100": lambda: _wide(1100, 2100, 6),
     "pulse": _pulse,
     "rmat-13007": lambda: gen.rmat(14, 12, seed=21, n=13007, m=13007 * 12),
     "rmat-17001": lambda: gen.rmat(15, 24, seed=22, n=17001, m=17001 * 24),
