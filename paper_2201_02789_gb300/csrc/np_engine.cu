@@ -482,12 +482,8 @@ int resolve_driver(const Plan& p, const np_config& cfg) {
   return p.mode == M_DEVICE_LAUNCH ? NP_DRIVER_CHUNK : NP_DRIVER_WHILE;
 }
 
-namespace {
-
-// A launch that may be scheduled while its predecessor on the stream is still
-// running (programmatic dependent launch); the kernel waits for it itself.
 cudaError_t launch_pdl(const void* fn, dim3 grid, dim3 block, void** args, cudaStream_t s, bool pdl,
-                       size_t smem = 0, int cluster = 0) {
+                       size_t smem, int cluster) {
   if (!pdl && !cluster) return cudaLaunchKernel(fn, grid, block, args, smem, s);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
@@ -511,7 +507,7 @@ cudaError_t launch_pdl(const void* fn, dim3 grid, dim3 block, void** args, cudaS
   return cudaLaunchKernelExC(&cfg, fn, args);
 }
 
-constexpr bool kPdl = NP_PDL != 0;
+namespace {
 
 AggSeg make_seg(const Plan& p, const Args& a, const Grids& g, bool level_mode) {
   AggSeg seg{};

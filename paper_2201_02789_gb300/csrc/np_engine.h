@@ -144,6 +144,12 @@ Grids grids_for(Engine& e, const Plan& p, const np_config& cfg, int64_t max_pare
 // AUTO resolved: chunks for the device-launch forms, a conditional while loop otherwise.
 int resolve_driver(const Plan& p, const np_config& cfg);
 
+// A launch that may be scheduled while its predecessor on the stream is still
+// running (programmatic dependent launch); the kernel waits for it itself.
+cudaError_t launch_pdl(const void* fn, dim3 grid, dim3 block, void** args, cudaStream_t s, bool pdl,
+                       size_t smem = 0, int cluster = 0);
+constexpr bool kPdl = NP_PDL != 0;
+
 np_status enqueue_pass(const Plan& p, Args a, const Grids& g, bool level_mode, int k, cudaStream_t s);
 // The two grids of a tessellation pass (Plan::points), on s; `mid`, if not
 // NULL, is recorded between them. The resident CTAs per SM of the count grid

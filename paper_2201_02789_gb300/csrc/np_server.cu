@@ -12,8 +12,8 @@
 // L0). After `levels_per_step` levels a histogram of the frontier counts each
 // slot's remaining vertices; a resident query with none left is finished and
 // its result is copied to the caller's array. All of one pool's step is a
-// single CUDA graph (admission table upload, slot reset, source push, the
-// levels, histogram, result copy, count read-back) on the pool's own stream.
+// single CUDA graph (admission table upload, admission, the levels, histogram,
+// result copy and read-back) on the pool's own stream.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -46,80 +46,80 @@ __device__ __forceinline__ const int* dctl_busy(const Ctl* c, int S) {
   return reinterpret_cast<const int*>(dctl_adm(c) + S);
 }
 
-// Resets the arrays of the slots admitted this step (blockIdx.y = admission).
-// SSSP pools keep the packed state (distance << 32 | append tag).
-__global__ void slot_reset_kernel(const Ctl* ctl, int kind, int lg, int* level, unsigned long long* dtag) {
+// The start of a step: the counts of the last one cleared, the slots admitted in
+// this one (blockIdx.y = admission) reset and their sources put into the
+// frontier of the current level. SSSP pools keep the packed state (distance <<
+// 32 | append tag).
+__global__ void slot_admit_kernel(LevelState* st, const Ctl* ctl, int S, int kind, int lg, int* level,
+                                  unsigned long long* dtag, int* fr0, int* fr1, unsigned long long* slot_out,
+                                  int* slot_L0, int* active) {
+  NP_PDL_ENTRY();
+  if (blockIdx.x == 0 && blockIdx.y == 0)
+    for (int q = threadIdx.x; q < S; q += blockDim.x) active[q] = 0;
   if ((int)blockIdx.y >= ctl->nadm) return;
-  const int slot = dctl_adm(ctl)[blockIdx.y].x;
+  const int4 e = dctl_adm(ctl)[blockIdx.y];
+  const int slot = e.x, src = e.y, L = st->base;
   const long long base = (long long)slot << lg;
   const int npad = 1 << lg;
   for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < npad; v += gridDim.x * blockDim.x) {
     if (kind == 0)
-      level[base + v] = -1;
+      level[base + v] = v == src ? L : -1;
     else
-      dtag[base + v] = 0xffffffff00000000ull;
+      dtag[base + v] = v == src ? 0ull : 0xffffffff00000000ull;
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    ((L & 1) ? fr1 : fr0)[atomicAdd(&st->count[L % 3], 1)] = (int)base + src;
+    slot_out[slot] = ((unsigned long long)(unsigned)e.w << 32) | (unsigned)e.z;
+    slot_L0[slot] = L;
   }
 }
 
-// Puts the admitted sources into the frontier of the current level.
-__global__ void slot_admit_kernel(LevelState* st, const Ctl* ctl, int kind, int lg, int* level,
-                                  unsigned long long* dtag, int* fr0, int* fr1, unsigned long long* slot_out,
-                                  int* slot_L0) {
-  __shared__ int c0, L;
-  const int nadm = ctl->nadm;
-  if (nadm <= 0) return;
-  if (threadIdx.x == 0) {
-    L = st->base;
-    c0 = st->count[L % 3];
-  }
-  __syncthreads();
-  int* fr = (L & 1) ? fr1 : fr0;
-  for (int i = threadIdx.x; i < nadm; i += blockDim.x) {
-    const int4 a = dctl_adm(ctl)[i];
-    const int id = (a.x << lg) | a.y;
-    if (kind == 0)
-      level[id] = L;
-    else
-      dtag[id] = 0ull;
-    fr[c0 + i] = id;
-    slot_out[a.x] = ((unsigned long long)(unsigned)a.w << 32) | (unsigned)a.z;
-    slot_L0[a.x] = L;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) st->count[L % 3] = c0 + nadm;
-}
-
-// active[q] = frontier entries of slot q at the current level; active[S] = level.
-__global__ void slot_histogram_kernel(const LevelState* st, const int* fr0, const int* fr1, int lg, int S,
+// active[q] += frontier entries of slot q at the level K past the step's first.
+__global__ void slot_histogram_kernel(const LevelState* st, int K, const int* fr0, const int* fr1, int lg, int S,
                                       int* active) {
+  NP_PDL_ENTRY();
   __shared__ int h[kMaxSlots];
-  for (int q = threadIdx.x; q < S; q += blockDim.x) h[q] = 0;
-  __syncthreads();
-  const int L = __ldcg(&st->base);
+  const int L = __ldcg(&st->base) + K;
   const int cnt = __ldcg(&st->count[L % 3]);
   const int* ids = (L & 1) ? fr1 : fr0;
+  if ((long long)blockIdx.x * blockDim.x >= cnt) return;
+  for (int q = threadIdx.x; q < S; q += blockDim.x) h[q] = 0;
+  __syncthreads();
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += gridDim.x * blockDim.x)
     atomicAdd(&h[__ldcg(&ids[i]) >> lg], 1);
   __syncthreads();
   for (int q = threadIdx.x; q < S; q += blockDim.x)
     if (h[q]) atomicAdd(&active[q], h[q]);
-  if (blockIdx.x == 0 && threadIdx.x == 0) active[S] = L;
 }
 
-// Copies every resident slot with no frontier entries left to its caller's array.
-__global__ void slot_retire_kernel(const Ctl* ctl, int S, const int* active, int kind, int lg, int n,
-                                   const int* level, const unsigned long long* dtag,
-                                   const unsigned long long* slot_out, const int* slot_L0) {
+// The end of a step: every resident slot with no frontier entries left is
+// copied to its caller's array, the level base moves on, and the counts and the
+// error word go to the pinned words that the host reads.
+__global__ void slot_retire_kernel(LevelState* st, int K, const Ctl* ctl, int S, const int* active, int kind, int lg,
+                                   int n, const int* level, const unsigned long long* dtag,
+                                   const unsigned long long* slot_out, const int* slot_L0, int* host) {
+  NP_PDL_ENTRY();
   const int slot = blockIdx.y;
-  if (!dctl_busy(ctl, S)[slot] || __ldcg(&active[slot]) != 0) return;
+  const int left = __ldcg(&active[slot]);
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    host[slot] = left;
+    if (slot == 0) {
+      const int L = st->base + K;
+      st->base = L;
+      host[S] = L;
+      host[S + 1] = (int)st->error;
+    }
+  }
+  if (!dctl_busy(ctl, S)[slot] || left != 0) return;
   const long long base = (long long)slot << lg;
-  const int L0 = slot_L0[slot];
+  const int L0 = __ldcg(&slot_L0[slot]);
+  void* out = reinterpret_cast<void*>(__ldcg(&slot_out[slot]));
   for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
     if (kind == 0) {
-      const int l = level[base + v];
-      reinterpret_cast<int*>(slot_out[slot])[v] = l >= 0 ? l - L0 : -1;
+      const int l = __ldcg(&level[base + v]);
+      static_cast<int*>(out)[v] = l >= 0 ? l - L0 : -1;
     } else {
-      reinterpret_cast<unsigned*>(slot_out[slot])[v] = (unsigned)(dtag[base + v] >> 32);
+      static_cast<unsigned*>(out)[v] = (unsigned)(__ldcg(&dtag[base + v]) >> 32);
     }
   }
 }
@@ -187,6 +187,12 @@ struct np_server {
 
 namespace {
 
+// What bounds a step of small levels is its chain of graph nodes: with slot
+// reset, admission, the clearing of the counts and the base advance in kernels
+// or nodes of their own and two read-back copies it had 15, now 10, nine of
+// them kernels that may start early (48 queries over four pools, 8 steps: 1303
+// -> 1069 us). The table is still uploaded by a copy: blocks of the admission
+// that read it from host memory themselves took 90 us a step.
 np_status build_pool_graph(np_server* sv, Pool& p) {
   Engine& e = sv->e;
   const BodyKernels& K = p.kind == 0 ? bfs_kernels() : sssp64_kernels();
@@ -211,34 +217,25 @@ np_status build_pool_graph(np_server* sv, Pool& p) {
     }
   }
   Grids gr = grids_for(e, plan, p.cfg, elems);
+  int lps = sv->levels_per_step;
+  void* hargs[] = {&p.ws.st, &lps, &a.fr0, &a.fr1, &p.lg, &p.S, &p.active};
+  void* rargs[] = {&p.ws.st, &lps, &p.d_ctl, &p.S, &p.active, &p.kind, &p.lg, &p.n, &p.level, &p.dtag, &p.slot_out,
+                   &p.slot_L0, &p.h_active};
   cudaStream_t cs = e.cap_stream;
   NP_CK(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
   np_status st = NP_OK;
   cudaError_t ce = cudaMemcpyAsync(p.d_ctl, p.h_ctl, ctl_bytes(p.S), cudaMemcpyHostToDevice, cs);
   if (ce == cudaSuccess) {
-    const int bx = blocks_for(1ll << p.lg, 256, 64);
-    slot_reset_kernel<<<dim3(bx, p.S), 256, 0, cs>>>(p.d_ctl, p.kind, p.lg, p.level, p.dtag);
-    slot_admit_kernel<<<1, 256, 0, cs>>>(p.ws.st, p.d_ctl, p.kind, p.lg, p.level, p.dtag, a.fr0, a.fr1, p.slot_out,
-                                         p.slot_L0);
+    slot_admit_kernel<<<dim3(blocks_for(1ll << p.lg, 256, 64), p.S), 256, 0, cs>>>(
+        p.ws.st, p.d_ctl, p.S, p.kind, p.lg, p.level, p.dtag, a.fr0, a.fr1, p.slot_out, p.slot_L0, p.active);
     ce = cudaGetLastError();
   }
-  if (ce == cudaSuccess) {
-    for (int k = 0; k < sv->levels_per_step && st == NP_OK; k++) st = enqueue_pass(plan, a, gr, true, k, cs);
-    if (st == NP_OK) st = enqueue_advance(p.ws.st, sv->levels_per_step, cs, true);
-  }
-  if (ce == cudaSuccess && st == NP_OK) ce = cudaMemsetAsync(p.active, 0, sizeof(int) * (size_t)(p.S + 1), cs);
-  if (ce == cudaSuccess && st == NP_OK) {
-    slot_histogram_kernel<<<std::max(1, std::min(e.sms * 2, blocks_for(elems))), 256, 0, cs>>>(
-        p.ws.st, a.fr0, a.fr1, p.lg, p.S, p.active);
-    const int bx = blocks_for(p.n, 256, 64);
-    slot_retire_kernel<<<dim3(bx, p.S), 256, 0, cs>>>(p.d_ctl, p.S, p.active, p.kind, p.lg, p.n, p.level, p.dtag,
-                                                       p.slot_out, p.slot_L0);
-    ce = cudaGetLastError();
-  }
+  for (int k = 0; k < lps && ce == cudaSuccess && st == NP_OK; k++) st = enqueue_pass(plan, a, gr, true, k, cs);
   if (ce == cudaSuccess && st == NP_OK)
-    ce = cudaMemcpyAsync(p.h_active, p.active, sizeof(int) * (size_t)(p.S + 1), cudaMemcpyDeviceToHost, cs);
-  if (ce == cudaSuccess && st == NP_OK)   // the pool's device error word
-    ce = cudaMemcpyAsync(p.h_active + p.S + 1, &p.ws.st->error, sizeof(unsigned), cudaMemcpyDeviceToHost, cs);
+    ce = launch_pdl((const void*)slot_histogram_kernel, dim3(std::max(1, std::min(e.sms * 2, blocks_for(elems)))),
+                    dim3(256), hargs, cs, kPdl);
+  if (ce == cudaSuccess && st == NP_OK)
+    ce = launch_pdl((const void*)slot_retire_kernel, dim3(blocks_for(p.n, 256, 64), p.S), dim3(256), rargs, cs, kPdl);
   cudaGraph_t graph = nullptr;
   cudaError_t ee = cudaStreamEndCapture(cs, &graph);
   if (st != NP_OK || ce != cudaSuccess || ee != cudaSuccess) {
