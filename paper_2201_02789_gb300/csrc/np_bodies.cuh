@@ -406,8 +406,7 @@ struct BezierBody {
     return (int)t;
   }
   // The same count without FP64 arithmetic where that is provably the same
-  // number (FP64 throughput is low on this GPU). When every coordinate is
-  // k * 2^-24 with 0 <= k < 2^24, the FP64 second difference, chord and their
+  // number. When every coordinate is k * 2^-24 with 0 <= k < 2^24, the FP64 second difference, chord and their
   // squared norms above are exact: s2 = S * 2^-48 and c2 = C * 2^-48 with
   // integers S < 2^53, C < 2^49. The exact t = 64 (S / C)^(1/4) then has
   // ceil(t) = the least m with m^4 C >= 2^24 S, found with 128-bit integers;
@@ -415,7 +414,7 @@ struct BezierBody {
   // rounded operations), so it has the same ceiling unless t^4 lies within a
   // relative 2^-40 of m^4 or (m-1)^4, where the FP64 sequence itself decides.
   // Other inputs also take the FP64 sequence.
-  __device__ static int point_count(const float* p) {
+  __device__ static int point_count_exact(const float* p) {
     unsigned k[6];
 #pragma unroll
     for (int i = 0; i < 6; i++) {
@@ -429,15 +428,6 @@ struct BezierBody {
     const unsigned long long C = (unsigned long long)(cx * cx) + (unsigned long long)(cy * cy);
     if (C == 0) return S > 0 ? 4096 : 4;
     if (S == 0) return 4;                                   // t = 0 exactly, in FP64 too
-    // FP32 first: S, C, their quotient and two square roots, each correctly
-    // rounded, put t within a relative 2.25 * 2^-24 (and a little) of its exact
-    // value, so unless an integer lies within 2^-21 of it the ceiling is settled
-    // (one random curve in some ten thousand goes on to the exact comparison)
-    {
-      const float t = 64.0f * sqrtf(sqrtf((float)S / (float)C));
-      const float up = ceilf(t * (1.0f + 0x1p-21f));
-      if (ceilf(t * (1.0f - 0x1p-21f)) == up) return up < 4.0f ? 4 : (up > 4096.0f ? 4096 : (int)up);
-    }
     using u128 = unsigned __int128;
     const u128 A = (u128)S << 24;                          // t^4 * C
     auto q4 = [&](unsigned long long m) -> u128 { const u128 m2 = (u128)(m * m); return m2 * m2 * C; };
@@ -453,6 +443,48 @@ struct BezierBody {
     const bool near = (hi - A) <= (hi >> 40) || (m > 1 && (A - lo) <= (lo >> 40));
     if (!exact_m || near) return point_count_fp64(p);
     return m < 4 ? 4 : (m > 4096 ? 4096 : (int)m);
+  }
+  // The same count from FP32 where that settles it (FP64 throughput is low on
+  // this GPU: a thread's FP64 sequence takes 5 us, and the 64-bit products of
+  // the exact form are slow too).
+  // With M the largest |coordinate|: the second difference is x0 - 2 x1 + x2
+  // as two exact sums and their low parts, so within 2^-24 |sx| + 2^-45 M;
+  // where its norm s is at least 2^-20 M that is below a relative 2^-23. The
+  // chord c has one rounding per component. Squares, sums, quotient and two
+  // square roots, each correctly rounded, put t = 64 sqrt(s / c) within a
+  // relative 2^-21.4, and the FP64 sequence (whose second difference is within
+  // 2^-50 M) is nearer still: unless an integer lies within 2^-20 of t, both
+  // have its ceiling. That leaves one random curve in some five thousand. A
+  // chord of 0 is exact. Where s is smaller, its bound |sx| + |sy| + 2^-40 M
+  // still settles t < 4.
+  __device__ static int point_count(const float* p) {
+    const float x0 = p[0], y0 = p[1], x1 = p[2], y1 = p[3], x2 = p[4], y2 = p[5];
+    const float M =
+        fmaxf(fmaxf(fmaxf(fabsf(x0), fabsf(y0)), fmaxf(fabsf(x1), fabsf(y1))), fmaxf(fabsf(x2), fabsf(y2)));
+    // a - 2 b + c by two-sums (Knuth, TAOCP 2, 4.2.2): no FMA may be made of them
+    auto second = [](float u, float v, float w) {
+      const float m = __fmul_rn(-2.0f, v);
+      const float h = __fadd_rn(u, m), hu = __fsub_rn(h, m);
+      const float l = __fadd_rn(__fsub_rn(u, hu), __fsub_rn(m, __fsub_rn(h, hu)));
+      const float g = __fadd_rn(h, w), gh = __fsub_rn(g, w);
+      const float k = __fadd_rn(__fsub_rn(h, gh), __fsub_rn(w, __fsub_rn(g, gh)));
+      return __fadd_rn(g, __fadd_rn(l, k));
+    };
+    const float sx = second(x0, x1, x2), sy = second(y0, y1, y2), cx = __fsub_rn(x2, x0), cy = __fsub_rn(y2, y0);
+    const float s2 = sx * sx + sy * sy, c2 = cx * cx + cy * cy;
+    // (no NaN or infinity passes, and nothing near the ends of the range)
+    if (((c2 >= 0x1p-60f && c2 <= 0x1p100f) || (cx == 0.0f && cy == 0.0f)) && M <= 0x1p50f) {
+      if (s2 >= 0x1p-60f && s2 >= 0x1p-40f * (M * M)) {
+        if (c2 == 0.0f) return 4096;
+        const float t = 64.0f * sqrtf(sqrtf(s2 / c2));
+        const float up = ceilf(t * (1.0f + 0x1p-20f));
+        if (ceilf(t * (1.0f - 0x1p-20f)) == up) return up < 4.0f ? 4 : (up > 4096.0f ? 4096 : (int)up);
+      } else {
+        const float s = fabsf(sx) + fabsf(sy) + 0x1p-40f * M;
+        if (s * s < 0x1p-17f * c2) return 4;
+      }
+    }
+    return point_count_exact(p);
   }
   __device__ static void count(const Args& a, int pid, int& base, int& N) {
     base = 0;
