@@ -8,6 +8,7 @@ const BodyKernels& bezier_kernels() {
     BodyKernels k = make_table<BezierBody>();
     k.points_count = (const void*)bezier_count;
     k.points = (const void*)bezier_points;
+    k.points_fused = (const void*)bezier_fused;
     return k;
   }();
   return t;

@@ -174,10 +174,15 @@ np_status fixed_pass(np_ctx* c, const Args& a0, const np_config& cfg, const Body
   Plan p = make_plan(K, cfg);
   Args a = a0;
   if (p.points) {
+    // (these launches could be captured, with workspace pointers that a later
+    // call may free: refused, as the graph launch below is on such a stream)
+    cudaStreamCaptureStatus cap;
+    NP_CK(cudaStreamIsCapturing(s, &cap));
+    if (cap != cudaStreamCaptureStatusNone) return NP_ERR_CUDA;
     const int occ = occupancy(c->e, p.parent, kPointBlock);
-    if (!c->e.profile) return enqueue_points(p, a, cfg.parent_grid, c->e.sms, occ, s);
+    if (!c->e.profile) return enqueue_points(p, a, cfg.parent_grid, c->e.sms, occ, kPdl, s);
     NP_CK(cudaEventRecord(c->e.ev[0], s));
-    NP_TRY(enqueue_points(p, a, cfg.parent_grid, c->e.sms, occ, s, c->e.ev[1]));
+    NP_TRY(enqueue_points(p, a, cfg.parent_grid, c->e.sms, occ, false, s, c->e.ev[1]));
     NP_CK(cudaEventRecord(c->e.ev[2], s));
     NP_CK(cudaEventSynchronize(c->e.ev[2]));
     float t01 = 0.f, t12 = 0.f;

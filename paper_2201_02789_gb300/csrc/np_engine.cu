@@ -391,6 +391,7 @@ Plan make_plan(const BodyKernels& K, const np_config& cfg) {
     if (K.points && form == NP_SERIAL_SPREAD) {
       p.parent = K.points_count;
       p.child = K.points;
+      p.points_fused = K.points_fused;
       p.child_idle = false;
       p.points = true;
     }
@@ -566,11 +567,8 @@ np_status enqueue_pass(const Plan& p, Args a, const Grids& g, bool level_mode, i
   return NP_OK;
 }
 
-// The count grid is launched after everything before it on the stream (it may
-// follow a launch that is not a kernel, and stream capture then has no
-// programmatic edge to make of it); the point grid may be scheduled early.
-np_status enqueue_points(const Plan& p, Args a, int parent_grid, int sms, int occ_count, cudaStream_t s,
-                         cudaEvent_t mid) {
+np_status enqueue_points(const Plan& p, Args a, int parent_grid, int sms, int occ_count, bool early,
+                         cudaStream_t s, cudaEvent_t mid) {
   const int tiles = (int)(((int64_t)a.count_fixed + kPointBlock - 1) / kPointBlock);
   const int per = kPointBlock / 32 * kPointCurves;   // curves of one point CTA
   // CTAs over the curves, whole tiles of them, and one for the totals unless the count grid takes those
@@ -580,7 +578,10 @@ np_status enqueue_points(const Plan& p, Args a, int parent_grid, int sms, int oc
   int pg = parent_grid > 0 ? parent_grid : occ_count * sms;
   if (pg > tiles) pg = tiles;
   void* args[] = {&a};
-  NP_CK(cudaLaunchKernel(p.parent, dim3(pg), dim3(kPointBlock), args, 0, s));
+  if (a.count_fixed <= kPointFused && parent_grid == 0 && !mid)
+    return from_cuda(launch_pdl(p.points_fused, dim3((unsigned)((a.count_fixed + per - 1) / per + 1)),
+                                dim3(kPointBlock), args, s, early));
+  NP_CK(launch_pdl(p.parent, dim3(pg), dim3(kPointBlock), args, s, early));
   if (mid) NP_CK(cudaEventRecord(mid, s));
   NP_CK(launch_pdl(p.child, dim3((unsigned)groups), dim3(kPointBlock), args, s, kPdl && !mid));
   return NP_OK;

@@ -41,6 +41,7 @@ struct BodyKernels {
   // as a count grid over the curves and a grid over their points
   const void* points_count;
   const void* points;
+  const void* points_fused;   // both in one, for few curves
 };
 
 const BodyKernels& bfs_kernels();

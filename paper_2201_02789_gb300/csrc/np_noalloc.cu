@@ -148,7 +148,7 @@ extern "C" np_status np_bezier_noalloc(const float* ctrl, int32_t ncurves, int32
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, plan.parent, kPointBlock, 0) != cudaSuccess || occ < 1)
       occ = 1;
     // (no bounded wait on this path: offsets[ncurves] is always the total)
-    return enqueue_points(plan, a, cfg->parent_grid, d.sms, occ, s);
+    return enqueue_points(plan, a, cfg->parent_grid, d.sms, occ, false, s);
   }
   const void* parent = plan.parent;
   const int pb = cfg->parent_block, cb = cfg->child_block;

@@ -23,8 +23,8 @@ namespace nestpar {
 // CTA waits for another one's offsets: with both in one kernel each group of
 // tiles waited for its look-back before it could store its first point, and a
 // CTA held 450-500 curves, too coarse to fill 152 SMs. Measured, one pass of
-// random curves (6.2 M and 25 M points, threshold 32 and none): 43.9 -> 16.4 us
-// and 64.8 -> 43.5 us; the point grid alone takes 34 us for 25 M points (200 MB
+// random curves (6.2 M and 25 M points, threshold 32 and none): 43.9 -> 15.1 us
+// and 64.8 -> 42.6 us; the point grid alone takes 34 us for 25 M points (200 MB
 // of stores, 30 us at the copy bandwidth; 68% of the issue slots).
 static_assert(kPointBlock % (kPointBlock / 32 * kPointCurves) == 0, "a point CTA's curves lie in one count tile");
 constexpr int kPointTile = kPointBlock;   // N <= 4096: an offset in the tile takes 20 bits
@@ -38,11 +38,39 @@ constexpr int kPointTile = kPointBlock;   // N <= 4096: an offset in the tile ta
 // cost the same: 12.6 + 34.4 us with the scan, 8.2 + 38.9 us without; at 256
 // tiles a pass takes 18.4 and 16.5 us.)
 
+// np_stats and the total from what the threads of one CTA counted.
+__device__ __forceinline__ void point_stats(const Args& a, unsigned items, unsigned serial, unsigned launched,
+                                            unsigned citems, unsigned cblocks, unsigned curves, unsigned total) {
+  __shared__ unsigned s_sum[6];
+  const int tid = (int)threadIdx.x;
+  if (tid < 6) s_sum[tid] = 0u;
+  __syncthreads();
+  const unsigned v[6] = {items, serial, launched, citems, cblocks, curves};
+#pragma unroll
+  for (int k = 0; k < 6; k++) {
+    const unsigned x = __reduce_add_sync(kFull, v[k]);
+    if ((tid & 31) == 0) atomicAdd(&s_sum[k], x);
+  }
+  __syncthreads();
+  if (tid == 0) {
+    LevelState* st = a.st;
+    for (int k = 0; k < S_N; k++) st->s[k] = 0ull;
+    st->s[S_ITEMS] = s_sum[0];
+    st->s[S_SERIAL] = s_sum[1];
+    st->s[S_LAUNCHP] = s_sum[2];
+    st->s[S_CITEMS] = s_sum[3];
+    st->s[S_CBLOCKS] = s_sum[4];
+    st->s[S_PARENTS] = s_sum[5];
+    st->body_iters = 0;
+    if ((long long)total > a.cap) st->error |= kErrCapacity;
+    a.offsets[a.count_fixed] = (int)total;
+  }
+}
+
 // Statistics and the total from the tiles' sums, by one CTA of kPointTile
 // threads; with `scan` the tiles' exclusive prefixes go to a.lb_incl as words.
 __device__ __forceinline__ void point_totals(const Args& a, int ntiles, bool scan) {
   __shared__ uint2 s_scan2[33];
-  __shared__ unsigned s_sum[6];
   const int tid = (int)threadIdx.x, count = a.count_fixed;
   const int T = a.threshold < 1 ? 1 : a.threshold;
   const bool never = a.threshold == INT_MAX;
@@ -58,7 +86,6 @@ __device__ __forceinline__ void point_totals(const Args& a, int ntiles, bool sca
     cblocks += x.x;
     curves += x.y;
   }
-  if (tid < 6) s_sum[tid] = 0u;
   unsigned e0, e1, total, u1;
   block_scan2(items, 0u, e0, e1, total, u1, s_scan2);
   const unsigned* tile0 = nullptr;
@@ -95,26 +122,7 @@ __device__ __forceinline__ void point_totals(const Args& a, int ntiles, bool sca
       e0 += __ldcg(&a.lb_agg[t]).x;
     }
   }
-  const unsigned v[6] = {items, serial, launched, citems, cblocks, curves};
-#pragma unroll
-  for (int k = 0; k < 6; k++) {
-    const unsigned x = __reduce_add_sync(kFull, v[k]);
-    if ((tid & 31) == 0) atomicAdd(&s_sum[k], x);
-  }
-  __syncthreads();
-  if (tid == 0) {
-    LevelState* st = a.st;
-    for (int k = 0; k < S_N; k++) st->s[k] = 0ull;
-    st->s[S_ITEMS] = s_sum[0];
-    st->s[S_SERIAL] = s_sum[1];
-    st->s[S_LAUNCHP] = s_sum[2];
-    st->s[S_CITEMS] = s_sum[3];
-    st->s[S_CBLOCKS] = s_sum[4];
-    st->s[S_PARENTS] = s_sum[5];
-    st->body_iters = 0;
-    if ((long long)total > a.cap) st->error |= kErrCapacity;
-    a.offsets[count] = (int)total;
-  }
+  point_stats(a, items, serial, launched, citems, cblocks, curves, total);
 }
 
 __global__ void __launch_bounds__(kPointTile, 4) bezier_count(Args a) {
@@ -161,6 +169,40 @@ __global__ void __launch_bounds__(kPointTile, 4) bezier_count(Args a) {
 // kPointCurves curves at once, one per lane (offset, N, the six products), and
 // then runs them one after the other from shuffles: 17 instructions per 32
 // points and 14 per curve.
+//
+// Lane l holds curve `i` = its warp's curve l % kPointCurves: id `pid` (-1: none),
+// offset and number of points.
+__device__ __forceinline__ void point_curves(const Args& a, int i, int pid, int base, int N) {
+  const int lane = (int)threadIdx.x & 31;
+  float ax = 0.f, ay = 0.f, bx = 0.f, by = 0.f, cx = 0.f, cy = 0.f;
+  if (pid >= 0) {
+    const float* c = a.b.ctrl + 6 * (size_t)pid;
+    const float nm1 = (float)(N - 1), r = 1.0f / (nm1 * nm1), r2 = 2.0f * r;
+    ax = __ldg(c) * r;
+    ay = __ldg(c + 1) * r;
+    bx = __ldg(c + 2) * r2;
+    by = __ldg(c + 3) * r2;
+    cx = __ldg(c + 4) * r;
+    cy = __ldg(c + 5) * r;
+    if (lane < kPointCurves) a.offsets[i] = base;
+  }
+  if (pid < 0 || (long long)base + N > a.cap) N = 0;   // (none, or it does not fit: skipped)
+  for (int q = 0; q < kPointCurves; q++) {
+    const int n = __shfl_sync(kFull, N, q);
+    float2* out = a.b.points + __shfl_sync(kFull, base, q) + lane;
+    const float x0 = __shfl_sync(kFull, ax, q), y0 = __shfl_sync(kFull, ay, q), x1 = __shfl_sync(kFull, bx, q),
+                y1 = __shfl_sync(kFull, by, q), x2 = __shfl_sync(kFull, cx, q), y2 = __shfl_sync(kFull, cy, q);
+    float j = (float)lane, k = (float)(n - 1 - lane);
+    for (int left = n - lane; left > 0; left -= 32) {
+      const float w0 = k * k, w1 = j * k, w2 = j * j;
+      *out = make_float2(w0 * x0 + w1 * x1 + w2 * x2, w0 * y0 + w1 * y1 + w2 * y2);
+      out += 32;
+      j += 32.0f;
+      k -= 32.0f;
+    }
+  }
+}
+
 __global__ void __launch_bounds__(256, 6) bezier_points(Args a) {
   NP_PDL_ENTRY();
   const int lane = (int)threadIdx.x & 31;
@@ -187,40 +229,101 @@ __global__ void __launch_bounds__(256, 6) bezier_points(Args a) {
   }
   const int first = ((int)blockIdx.x * ((int)blockDim.x >> 5) + ((int)threadIdx.x >> 5)) * kPointCurves;
   const int i = first + (lane & (kPointCurves - 1));
-  int base = 0, N = 0;
-  float ax = 0.f, ay = 0.f, bx = 0.f, by = 0.f, cx = 0.f, cy = 0.f;
+  int base = 0, N = 0, pid = -1;
   if (i < count) {
     const unsigned w = (unsigned)__ldcg(&a.boff[i]);
-    const int pid = a.ids ? __ldcg(&a.ids[i]) : i;
-    if (pid >= 0) {
-      base = (int)(before + (w >> 12));
-      N = (int)(w & 4095u) + 1;
-      const float* c = a.b.ctrl + 6 * (size_t)pid;
-      const float nm1 = (float)(N - 1), r = 1.0f / (nm1 * nm1), r2 = 2.0f * r;
-      ax = __ldg(c) * r;
-      ay = __ldg(c + 1) * r;
-      bx = __ldg(c + 2) * r2;
-      by = __ldg(c + 3) * r2;
-      cx = __ldg(c + 4) * r;
-      cy = __ldg(c + 5) * r;
-      if (lane < kPointCurves) a.offsets[i] = base;
-      if ((long long)base + N > a.cap) N = 0;   // (does not fit: skipped)
-    }
+    pid = a.ids ? __ldcg(&a.ids[i]) : i;
+    base = (int)(before + (w >> 12));
+    N = (int)(w & 4095u) + 1;
   }
-  for (int q = 0; q < kPointCurves; q++) {
-    const int n = __shfl_sync(kFull, N, q);
-    float2* out = a.b.points + __shfl_sync(kFull, base, q) + lane;
-    const float x0 = __shfl_sync(kFull, ax, q), y0 = __shfl_sync(kFull, ay, q), x1 = __shfl_sync(kFull, bx, q),
-                y1 = __shfl_sync(kFull, by, q), x2 = __shfl_sync(kFull, cx, q), y2 = __shfl_sync(kFull, cy, q);
-    float j = (float)lane, k = (float)(n - 1 - lane);
-    for (int left = n - lane; left > 0; left -= 32) {
-      const float w0 = k * k, w1 = j * k, w2 = j * j;
-      *out = make_float2(w0 * x0 + w1 * x1 + w2 * x2, w0 * y0 + w1 * y1 + w2 * y2);
-      out += 32;
-      j += 32.0f;
-      k -= 32.0f;
+  point_curves(a, i, pid, base, N);
+}
+
+// Up to kPointFused curves: one grid in place of the two. Each CTA counts the
+// curves before its own itself (two a thread at 512), and so does the CTA for
+// the totals. What bounds it is the launch and one chain of control points,
+// counts and stores. Passes of 1, 64 and 300 curves one after the other: 2.5,
+// 3.6 and 4.3 us on the device (4.2, 5.2 and 5.6 with two grids), 4.7 us a call
+// on the host (6.1); at 1000 curves the two take the same, at 2048 one takes
+// 8.2 us and two 6.0.
+__global__ void __launch_bounds__(kPointBlock, 4) bezier_fused(Args a) {
+  NP_PDL_ENTRY();
+  const int tid = (int)threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int count = a.count_fixed;
+  const int c0 = (int)blockIdx.x * (kPointBlock / 32 * kPointCurves);   // the CTA's first curve
+  auto points_of = [&](int i, int& pid) {
+    int base = 0, N = 0;
+    pid = a.ids ? __ldcg(&a.ids[i]) : i;
+    if (pid >= 0) BezierBody::count(a, pid, base, N);
+    return N;
+  };
+  if (c0 >= count) {   // (the one CTA beyond the curves)
+    __shared__ uint2 s_scan2[33];
+    const int T = a.threshold < 1 ? 1 : a.threshold;
+    unsigned items = 0, serial = 0, launched = 0, citems = 0, cblocks = 0, curves = 0;
+    auto tally = [&](int i, long long& at, long long cap) {
+      int pid;
+      const int N = points_of(i, pid);
+      if (pid < 0) return;
+      curves++;
+      at += N;
+      if (at > cap) return;   // (does not fit: no children)
+      items += (unsigned)N;
+      if (a.threshold != INT_MAX && N >= T) {
+        launched++;
+        citems += (unsigned)N;
+        cblocks += (unsigned)ceil_div(ceil_div(N, a.child_block), a.cfactor);
+      } else {
+        serial++;
+      }
+    };
+    long long at = 0;
+#pragma unroll 4
+    for (int i = tid; i < count; i += kPointBlock) tally(i, at, LLONG_MAX);
+    unsigned e0, e1, total, u1;
+    block_scan2(items, 0u, e0, e1, total, u1, s_scan2);
+    if ((long long)total > a.cap) {
+      // again, in order: a run of curves per thread
+      const int per = ceil_div(count, kPointBlock), i0 = min(tid * per, count), i1 = min(i0 + per, count);
+      unsigned run = 0;
+      int pid;
+#pragma unroll 1
+      for (int i = i0; i < i1; i++) run += (unsigned)points_of(i, pid);
+      unsigned t1;
+      __syncthreads();
+      block_scan2(run, 0u, e0, e1, t1, u1, s_scan2);
+      items = serial = launched = citems = cblocks = curves = 0;
+      at = e0;
+#pragma unroll 1
+      for (int i = i0; i < i1; i++) tally(i, at, a.cap);
     }
+    point_stats(a, items, serial, launched, citems, cblocks, curves, total);
+    return;
   }
+  unsigned before = 0;
+  int pid = -1;
+#pragma unroll 4
+  for (int i = tid; i < c0; i += kPointBlock) before += (unsigned)points_of(i, pid);
+  before = __reduce_add_sync(kFull, before);
+  const int i = c0 + wid * kPointCurves + (lane & (kPointCurves - 1));
+  pid = -1;
+  const int N = i < count ? points_of(i, pid) : 0;
+  int incl = N;
+#pragma unroll
+  for (int d = 1; d < kPointCurves; d *= 2) {
+    const int o = __shfl_up_sync(kFull, incl, d, kPointCurves);
+    if ((lane & (kPointCurves - 1)) >= d) incl += o;
+  }
+  __shared__ unsigned s_before[kPointBlock / 32], s_own[kPointBlock / 32];
+  if (lane == kPointCurves - 1) {
+    s_before[wid] = before;
+    s_own[wid] = (unsigned)incl;
+  }
+  __syncthreads();
+  unsigned base = (unsigned)(incl - N);
+#pragma unroll
+  for (int k = 0; k < kPointBlock / 32; k++) base += s_before[k] + (k < wid ? s_own[k] : 0u);
+  point_curves(a, i, pid, (int)base, N);
 }
 
 }  // namespace nestpar

@@ -1,5 +1,6 @@
 """The tessellation's count and point grids at the edges of their tiles (256 curves, 64 per
-point CTA, 1024 tiles summed by the point CTAs themselves), with parent subsets and a capacity
+point CTA, 1024 tiles summed by the point CTAs themselves, one grid for both up to 512 curves),
+with parent subsets and a capacity
 that falls inside a tile. Offsets exact; points |g - r| <= 1e-5 max(|r|, 1) as everywhere
 (three exact integer weights times products rounded twice: below 1e-6)."""
 import numpy as np
@@ -33,7 +34,7 @@ def _few_points(n):
     return np.ascontiguousarray(out)
 
 
-@pytest.mark.parametrize("nc", [1, 8, 63, 64, 65, 255, 256, 257, 512, 4097, 262144, 262145, 300001])
+@pytest.mark.parametrize("nc", [1, 8, 63, 64, 65, 255, 256, 257, 511, 512, 513, 4097, 262144, 262145, 300001])
 def test_tile_edges(ctx, nc):
     ctrl = _few_points(nc) if nc > 10000 else gen.bezier_curves(nc, seed=52)
     ref_off, ref_pts = oracle.bezier(ctrl)
@@ -48,7 +49,7 @@ def test_tile_edges(ctx, nc):
         assert st["launch_parents"] == big and st["serial_parents"] == nc - big
 
 
-@pytest.mark.parametrize("nc", [700, 262500])
+@pytest.mark.parametrize("nc", [301, 500, 700, 262500])
 def test_capacity_inside_a_tile(ctx, nc):
     ctrl = _few_points(nc)
     ref_off, ref_pts = oracle.bezier(ctrl)
@@ -85,3 +86,48 @@ def test_parent_subset_with_padding(ctx):
     for k in np.flatnonzero(ids >= 0)[::7]:
         for j in (0, counts[k] - 1):
             assert bezier_tolerance_ok(p[first[k] + j], oracle.bezier_point(ctrl[ids[k]], counts[k], j))[0]
+
+
+@pytest.mark.parametrize("count", [1, 64, 65, 300, 512])
+def test_padded_parents_in_one_grid(ctx, count):
+    ctrl = gen.bezier_curves(600, seed=54)
+    ids = np.random.default_rng(count).permutation(600)[:count].astype(np.int32)
+    ids[::5] = -1
+    keep = ids >= 0
+    n_of = np.array([oracle.bezier_count(ctrl[i]) if i >= 0 else 0 for i in ids])
+    first = np.concatenate([[0], np.cumsum(n_of)])
+    c_d, id_d = torch.from_numpy(ctrl).cuda(), torch.from_numpy(ids).cuda()
+    for cap in (int(first[-1]), int(first[-1]) // 2):
+        off = torch.full((count + 1,), -7, dtype=torch.int32, device="cuda:0")
+        pts = torch.full((int(first[-1]) + 1, 2), float("nan"), dtype=torch.float32, device="cuda:0")
+        body = npb.np_body(kind=npb.NP_BODY_BEZIER_EVAL, ctrl=c_d.data_ptr(), offsets=off.data_ptr(),
+                           points=pts.data_ptr(), cap=cap)
+        status, st = npb.np_run_nested(ctx.handle, npb.np_parents(id_d.data_ptr(), count), npb.NP_COUNT_BEZIER, None,
+                                       body, npb.config("tca"), stats=True, check=False)
+        assert status == (npb.NP_OK if first[-1] <= cap else npb.NP_ERR_CAPACITY)
+        o, p = off.cpu().numpy(), pts.cpu().numpy()
+        np.testing.assert_array_equal(o[:-1][keep], first[:-1][keep])
+        assert (o[:-1][~keep] == -7).all() and o[-1] == first[-1]
+        fits = keep & (first[1:] <= cap)
+        assert st["parents"] == keep.sum() and st["items"] == n_of[fits].sum()
+        assert st["launch_parents"] == (n_of[fits] >= 32).sum()
+        for k in np.flatnonzero(keep):
+            row = p[first[k]:first[k + 1]]
+            if fits[k]:
+                ref = np.array([oracle.bezier_point(ctrl[ids[k]], n_of[k], j) for j in range(n_of[k])])
+                assert bezier_tolerance_ok(row, ref)[0]
+            else:
+                assert np.isnan(row).all()
+
+
+def test_refused_under_capture(ctx):
+    """A context's workspace may be freed by a later call, so its passes are not captured."""
+    ctrl = torch.from_numpy(gen.bezier_curves(700, seed=55)).cuda()
+    off = torch.empty(701, dtype=torch.int32, device="cuda:0")
+    pts = torch.empty(200000, 2, dtype=torch.float32, device="cuda:0")
+    npb.np_bezier(ctx.handle, ctrl, 700, off, pts, 200000)
+    torch.cuda.synchronize()
+    g, s = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    with torch.cuda.graph(g, stream=s):
+        off.zero_()
+        assert npb.np_bezier(ctx.handle, ctrl, 700, off, pts, 200000, check=False) == npb.NP_ERR_CUDA
