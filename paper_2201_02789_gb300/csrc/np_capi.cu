@@ -168,17 +168,19 @@ np_status solve_multi(np_ctx* c, int kind, const np_csr* g, int nsrc, const int3
   return finish(c->e, c->w, s, stats);
 }
 
-// One fixed pass over an explicit parent set.
+// One fixed pass over an explicit parent set; acc[0, nacc) is cleared first.
 np_status fixed_pass(np_ctx* c, const Args& a0, const np_config& cfg, const BodyKernels& K, int count,
-                     cudaStream_t s) {
+                     cudaStream_t s, unsigned long long* acc = nullptr, int nacc = 0) {
   Plan p = make_plan(K, cfg);
   Args a = a0;
-  if (p.points) {
+  if (p.mode != M_DEVICE_LAUNCH) {
     // (these launches could be captured, with workspace pointers that a later
-    // call may free: refused, as the graph launch below is on such a stream)
+    // call may free: refused, as a graph launch is on such a stream)
     cudaStreamCaptureStatus cap;
     NP_CK(cudaStreamIsCapturing(s, &cap));
     if (cap != cudaStreamCaptureStatusNone) return NP_ERR_CUDA;
+  }
+  if (p.points) {
     const int occ = occupancy(c->e, p.parent, kPointBlock);
     if (!c->e.profile) return enqueue_points(p, a, cfg.parent_grid, c->e.sms, occ, kPdl, s);
     NP_CK(cudaEventRecord(c->e.ev[0], s));
@@ -198,7 +200,7 @@ np_status fixed_pass(np_ctx* c, const Args& a0, const np_config& cfg, const Body
   Grids g = grids_for(c->e, p, cfg, count);
   if (c->e.profile) {
     NP_CK(cudaEventRecord(c->e.ev[0], s));
-    init_fixed_kernel<<<1, 1, 0, s>>>(c->w.st);
+    init_fixed_kernel<<<1, 256, 0, s>>>(c->w.st, acc, nacc);
     NP_CK(cudaGetLastError());
     NP_CK(cudaEventRecord(c->e.ev[3], s));
     NP_CK(cudaEventSynchronize(c->e.ev[3]));
@@ -208,35 +210,13 @@ np_status fixed_pass(np_ctx* c, const Args& a0, const np_config& cfg, const Body
     c->e.prof.other_launches += 1;
     return profiled_pass(c->e, c->w, p, a, g, false, s);
   }
-  if (p.mode == M_DEVICE_LAUNCH) {
-    // device launches are joined by stream order only (a graph node does not
-    // wait for the grids it launches): no graph for these forms
-    init_fixed_kernel<<<1, 1, 0, s>>>(c->w.st);
-    NP_CK(cudaGetLastError());
-    return enqueue_pass(p, a, g, false, 0, s);
-  }
-  std::string key = graph_key("fixed", p, a, g, 1);
-  auto it = c->w.graphs.find(key);
-  cudaGraphExec_t exec = nullptr;
-  if (it != c->w.graphs.end()) {
-    exec = it->second.exec;
-  } else {
-    NP_CK(cudaStreamBeginCapture(c->e.cap_stream, cudaStreamCaptureModeThreadLocal));
-    init_fixed_kernel<<<1, 1, 0, c->e.cap_stream>>>(c->w.st);
-    cudaError_t le = cudaGetLastError();
-    np_status st = le == cudaSuccess ? enqueue_pass(p, a, g, false, 0, c->e.cap_stream) : from_cuda(le);
-    cudaGraph_t graph = nullptr;
-    cudaError_t e = cudaStreamEndCapture(c->e.cap_stream, &graph);
-    if (st != NP_OK) {
-      if (graph) cudaGraphDestroy(graph);
-      return st;
-    }
-    NP_CK(e);
-    st = cache_graph(c->w, key, graph, &exec);
-    if (st != NP_OK) return st;
-  }
-  NP_CK(cudaGraphLaunch(exec, s));
-  return NP_OK;
+  // Launches of their own: as a graph the same three kernels cost its launch
+  // and, for each new set of buffers, its instantiation (triangles of 500, 3000
+  // and 131,072 vertices: 20.8 -> 16.8, 29.2 -> 26.0, 297 -> 294 us). The first
+  // one waits in stream order: scheduled early it cost the large pass 7 us.
+  init_fixed_kernel<<<1, 256, 0, s>>>(c->w.st, acc, nacc);
+  NP_CK(cudaGetLastError());
+  return enqueue_pass(p, a, g, false, 0, s);
 }
 
 np_status stage_bytes(np_ctx* c, size_t bytes) {
@@ -390,7 +370,6 @@ np_status np_triangles(np_ctx* c, const np_csr* dag, uint64_t* count, const np_c
   cudaStream_t s = (cudaStream_t)stream;
   if (!c->tri) NP_CK(cudaMalloc(&c->tri, sizeof(unsigned long long) * kTcSlots));
   NP_TRY(ws_ensure(c->w, dag->n));
-  NP_CK(cudaMemsetAsync(c->tri, 0, sizeof(unsigned long long) * kTcSlots, s));
   Args a;
   base_args(c->w, *cfg, a);
   a.count_fixed = dag->n;
@@ -400,9 +379,11 @@ np_status np_triangles(np_ctx* c, const np_csr* dag, uint64_t* count, const np_c
   a.b.row_ptr = dag->row_ptr;
   a.n_vertices = dag->n;
   a.b.acc = c->tri;
-  NP_TRY(fixed_pass(c, a, *cfg, tc_kernels(), dag->n, s));
-  sum_u64_kernel<<<1, 256, 0, s>>>(c->tri, kTcSlots, reinterpret_cast<unsigned long long*>(count), 0);
-  NP_CK(cudaGetLastError());
+  int slots = kTcSlots, add = 0;
+  NP_TRY(fixed_pass(c, a, *cfg, tc_kernels(), dag->n, s, c->tri, slots));
+  void* args[] = {&c->tri, &slots, &count, &add};
+  NP_CK(launch_pdl((const void*)sum_u64_kernel, dim3(1), dim3(256), args, s,
+                   kPdl && make_plan(tc_kernels(), *cfg).mode != M_DEVICE_LAUNCH));
   return finish(c->e, c->w, s, stats);
 }
 

@@ -75,7 +75,10 @@ __global__ void init_solve_kernel(LevelState* st, int kind, int n, int src, int*
   }
 }
 
-__global__ void init_fixed_kernel(LevelState* st) { reset_slots(st); }
+__global__ void init_fixed_kernel(LevelState* st, unsigned long long* acc, int nacc) {
+  for (int i = (int)threadIdx.x; i < nacc; i += (int)blockDim.x) acc[i] = 0ull;
+  if (threadIdx.x == 0) reset_slots(st);
+}
 
 __global__ void fill_unreached_kernel(int kind, long long total, int* level, unsigned* dist, int* stamp) {
   const long long stride = (long long)gridDim.x * blockDim.x;
@@ -125,6 +128,7 @@ __global__ void csr_check_kernel(const int* row_ptr, const int* col, int n, long
 }
 
 __global__ void sum_u64_kernel(const unsigned long long* part, int n, unsigned long long* out, int accumulate) {
+  NP_PDL_ENTRY();
   __shared__ unsigned long long s[32];
   unsigned long long v = 0;
   for (int i = threadIdx.x; i < n; i += blockDim.x) v += part[i];

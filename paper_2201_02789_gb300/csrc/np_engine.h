@@ -197,7 +197,8 @@ np_status launch_level_loop(Engine& e, const Plan& p, const Args& a, const np_co
 // ---- device-side initialisation kernels (np_engine.cu)
 __global__ void init_solve_kernel(LevelState* st, int kind, int n, int src, int* level, unsigned* dist, int* stamp,
                                   int* fr0, int max_levels);
-__global__ void init_fixed_kernel(LevelState* st);
+// Before a fixed pass: the level header and acc[0, nacc) cleared (one block).
+__global__ void init_fixed_kernel(LevelState* st, unsigned long long* acc, int nacc);
 // Multi-source start: every element of level/dist/stamp[0, total) to its unreached value.
 __global__ void fill_unreached_kernel(int kind, long long total, int* level, unsigned* dist, int* stamp);
 // Then the sources (ids into those arrays) become level 0 / distance 0 and the first frontier.

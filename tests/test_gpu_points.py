@@ -8,7 +8,7 @@ import pytest
 import torch
 
 import oracle
-from gpu_util import bezier
+from gpu_util import DevGraph, bezier
 from invariants import bezier_tolerance_ok
 from paper_2201_02789_gb300 import gen
 from paper_2201_02789_gb300 import nestpar as npb
@@ -126,8 +126,29 @@ def test_refused_under_capture(ctx):
     off = torch.empty(701, dtype=torch.int32, device="cuda:0")
     pts = torch.empty(200000, 2, dtype=torch.float32, device="cuda:0")
     npb.np_bezier(ctx.handle, ctrl, 700, off, pts, 200000)
+    dg, count = DevGraph(gen.rmat(8, 4, seed=3)), torch.zeros(1, dtype=torch.int64, device="cuda:0")
+    npb.np_triangles(ctx.handle, dg.csr, count)
     torch.cuda.synchronize()
     g, s = torch.cuda.CUDAGraph(), torch.cuda.Stream()
     with torch.cuda.graph(g, stream=s):
         off.zero_()
         assert npb.np_bezier(ctx.handle, ctrl, 700, off, pts, 200000, check=False) == npb.NP_ERR_CUDA
+        assert npb.np_bezier(ctx.handle, ctrl, 700, off, pts, 200000, npb.config("nodp"),
+                             check=False) == npb.NP_ERR_CUDA
+        assert npb.np_triangles(ctx.handle, dg.csr, count, check=False) == npb.NP_ERR_CUDA
+
+
+@pytest.mark.parametrize("gran", ["none", "warp", "block", "multiblock", "grid_device"])
+def test_after_device_launched_children(ctx, gran):
+    """A pass whose grid may be scheduled early still waits for the children that the pass before it
+    launched from the device: both write the same points."""
+    a, b = (torch.from_numpy(gen.bezier_curves(n, seed=n)).cuda() for n in (3000, 300))
+    off = torch.empty(3001, dtype=torch.int32, device="cuda:0")
+    pts = torch.empty(600000, 2, dtype=torch.float32, device="cuda:0")
+    npb.np_bezier(ctx.handle, b, 300, off, pts, 600000)
+    total = int(off[300].item())
+    ref = pts[:total].clone()
+    for _ in range(5):
+        npb.np_bezier(ctx.handle, a, 3000, off, pts, 600000, npb.config("tca", granularity=gran, threshold=0))
+        npb.np_bezier(ctx.handle, b, 300, off, pts, 600000)
+        assert int(off[300].item()) == total and torch.equal(pts[:total], ref)
