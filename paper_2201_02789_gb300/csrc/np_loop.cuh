@@ -113,7 +113,9 @@ namespace nestpar {
 // first one too large, or an empty frontier. It runs once before the loop and
 // at the end of every body in place of the condition kernel: it moves the base
 // on by the body's K levels, runs what it can, and sets the loop's condition
-// (iterations counted and capped only at the end of a body).
+// (iterations counted and capped only at the end of a body). BFS only: the
+// packed SSSP has sssp_cluster in its place, and a BFS of one traversal starts
+// with bfs_first_levels instead (both below).
 #ifndef NP_SMALL_ITEMS
 #define NP_SMALL_ITEMS 16384
 #endif

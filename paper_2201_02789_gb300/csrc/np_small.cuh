@@ -134,14 +134,19 @@ constexpr int kClEntries = kClPull + kClFar + kClWide;
 constexpr int kFarList = kClFar * kClThreads;
 constexpr int kWideList = 64;                   // wide parents of one CTA (16 of them: kClWide * kClThreads slices)
 constexpr int kWideItems = 2048;
-// Children of one CTA in a round beyond which it defers the rest, and of all
-// published parents together, beyond which the grids take over; first for a graph with no more vertices than the
-// frontier limit (it cannot outgrow the cluster, and the grids' fixed cost per
-// level is then what counts), then for a larger one.
-constexpr int kClUnfiltered = 1024;
-constexpr int kClItemsSmall = 32768, kClItemsLarge = 4096;
-constexpr unsigned kStartItems = 8192;          // of a first frontier of at most 32 vertices of a larger graph
+// Children of one CTA in a round beyond which it defers the rest; where half of
+// the CTAs have so many, the grids take over (65,536 children or so: about what
+// a round and a level of the grids both take 25 us for). Without that the
+// cluster went on through such frontiers a budget at a time: R-MAT graphs of
+// 20,000 and 40,000 vertices with 16 and 8 edges each took 232 and 243 us
+// instead of 153 and 168 (184 and 196 before the cluster loop).
+constexpr int kClItems = 4096;
+// Children of all published parents together beyond which the grids take over;
+// first for a graph with no more vertices than the frontier limit (it cannot
+// outgrow the cluster), then for a larger one.
 constexpr unsigned kWideSmall = 524288u, kWideLarge = 32768u;
+constexpr unsigned kStartItems = 8192;          // of a first frontier of at most 32 vertices of a larger graph
+constexpr int kClUnfiltered = 1024;
 constexpr int kWinHigh = 2048;
 constexpr unsigned kNoCut = 0xffffffffu;
 constexpr size_t kClusterSmem =
@@ -182,7 +187,6 @@ __global__ void __launch_bounds__(kClThreads) sssp_cluster(Args a, cudaGraphCond
   unsigned long long n_par = 0, n_items = 0, n_serial = 0, n_levels = 0, n_push = 0;
   int total = count0, wide_all = 0;   // entries and wide parents of all CTAs
   const bool fits = a.n_vertices <= limit;
-  const int item_max = fits ? kClItemsSmall : kClItemsLarge;
   const unsigned wide_max = fits ? kWideSmall : kWideLarge;
   bool ran = count0 > 0 && count0 <= limit && L < max_levels;
   if (ran && !fits && count0 <= 32) {
@@ -240,6 +244,7 @@ __global__ void __launch_bounds__(kClThreads) sssp_cluster(Args a, cudaGraphCond
       // the grids take over: the frontier, or its children, too many for a cluster
       if (total > limit || __any_sync(kFull, mine > kClStage) || --rounds_left <= 0) break;
       if (wide_all > 0 && __reduce_add_sync(kFull, min((unsigned)h0.z, 1u << 26)) > wide_max) break;
+      if (2 * __popc(__ballot_sync(kFull, h0.w != 0)) >= nc) break;
       if (total > high && (cut != kNoCut || (prev > 0 && total >= prev && total < 2 * prev))) {
         // the middle of the last round's distances
         const int4 h1 = lane < nc ? s_hdr[cur][lane][1] : make_int4(-1, 0, 0, 0);
@@ -408,7 +413,7 @@ __global__ void __launch_bounds__(kClThreads) sssp_cluster(Args a, cudaGraphCond
       int at = 0;
       if (sum > 512u && lane == 0) at = atomicAdd(&s_budget, (int)sum);
       at = __shfl_sync(kFull, at, 0);
-      if (at + (int)sum > item_max) {
+      if (at + (int)sum > kClItems) {
         if (lane == 0) s_over = 1;
 #pragma unroll
         for (int r = 0; r < kClPull; r++) {
