@@ -92,12 +92,9 @@ WORKLOADS = {
 
 # per-workload values of the aggregated form's knobs, from threshold x cfactor x child-block
 # sweeps on GB300 (the paper also tunes T and CF per benchmark); other workloads use the defaults
-TUNED = {# tessellation: a threshold above every count, so that each curve's points run in its parent
-         # warp (a whole warp per curve of 32 points or more) and no child grid is launched: 35 against
-         # 42 us with the aggregated child grid below (BT_CHILD_GRID); 512-thread parent CTAs make the
-         # output-offset look-back groups 16 tiles long
+TUNED = {# tessellation: its count and point grids run whatever the threshold (which decides only what
+         # the statistics report as launched)
          "bt64k": dict(threshold=2**31 - 1, parent_block=512),
-         # (BT-256K: 448-thread parent CTAs, 66.7 against 68.7 us at 512; BT-64K the same at both)
          "bt256k": dict(threshold=2**31 - 1, parent_block=448),
          "tc-rmat17": dict(threshold=8, child_block=32, cfactor=1),
          # SSSP: every grid level's children only reduce and a sweep over the vertex state forms the
@@ -109,15 +106,15 @@ TUNED = {# tessellation: a threshold above every count, so that each curve's poi
          "bfs-rmat20": dict(sweep_parents=0),
          # road grid (out-degree <= 8): a threshold above every degree launches nothing, so no child
          # grid runs at any level; appending frontiers (a sweep reads the whole state for a frontier
-         # of about a tenth of it); 16 levels per while body over its 900 levels: 9.5 against 13.2 ms
-         # with the defaults
+         # of about a tenth of it); 16 levels per while body: 9.5 against 13.2 ms with the defaults
+         # where every level runs its grids, 4.3 ms with both in the SSSP cluster
          "road": dict(threshold=2**31 - 1, sweep_parents=0, unroll=16)}
 # the tessellation's best form with an aggregated child grid: T 32 (the default), 32-thread child
 # blocks of 4 original blocks, 512-thread parent CTAs spreading the serialised points over the CTA
-# (serial 2: NP_SERIAL_BLOCK); timed beside the headline
+# (serial 2: NP_SERIAL_BLOCK); timed beside the headline (39 against 15 us)
 BT_CHILD_GRID = dict(parent_block=512, child_block=32, cfactor=4, serial=2)
-# (the 4096-vertex graph, latency-bound, runs almost every level in the while driver's one-CTA
-# small-level loop: 115 us, against 150 us on the persistent level loop with 8 CTAs)
+# (the 4096-vertex graph, latency-bound, runs its levels in one CTA before the while loop, with
+# visited bits in shared memory: 55 us, against 171 us on the persistent level loop with 8 CTAs)
 
 
 def log(*a):
@@ -729,11 +726,11 @@ def run_ours(args, ws, rank, local):
             torch.distributed.destroy_process_group()
         return
 
-    # kernels launched per solve: graph solves launch init (+ the small-level loop once before
+    # kernels launched per solve: graph solves launch init (+ a small-level loop once before
     # the while loop) + per while-body iteration `unroll` x (parent, child[, sweep]) + the
     # condition kernel (the small-level loop); a tessellation launches init, parent and child
     # (no child when the threshold launches nothing and no children are packed for it)
-    # a tessellation with spread children launches its count and point grids
+    # (with spread children its count and point grids; one grid up to 512 curves)
     if wl["kind"] == "bezier":
         if cfg.serial == npb.NP_SERIAL_SPREAD:
             per_solve = 2
@@ -794,6 +791,8 @@ def run_ours(args, ws, rank, local):
     # serial children (whose child grid is child_agg_pack)
     cta = cfg.serial in (npb.NP_SERIAL_BLOCK, npb.NP_SERIAL_PACKED)
     child_name = "child_agg_pack" if cfg.serial == npb.NP_SERIAL_PACKED else "child_agg"
+    if wl["kind"] == "tc" and cfg.serial == npb.NP_SERIAL_SPREAD:
+        child_name = "tc_child"
     kernels = {child_name: (prof["child_ms"], prof["child_launches"], kb["child"]),
                ("parent_cta" if cta else "parent_warp"): (prof["parent_ms"], prof["parent_launches"], kb["parent"])}
     if wl["kind"] == "bezier" and cfg.serial == npb.NP_SERIAL_SPREAD:
