@@ -198,24 +198,27 @@ __global__ void __launch_bounds__(kClThreads) sssp_cluster(Args a, cudaGraphCond
     if (id >= 0) Body::count(a, id, row, deg);
     ran = __reduce_add_sync(kFull, min((unsigned)deg, 1u << 24)) <= kStartItems;
   }
-  if (ran) {
-    if (tid == 0) {
-      if (rank == 0) st->small_n = 0;
-      s_n = 0;
-      s_nwide = 0;
-      s_ndefer = 0;
-      s_far_n = 0;
-      s_par = 0;
-      s_budget = 0;
-      s_over = 0;
-      s_wide_items = 0u;
-      s_tot = 0ull;
-      s_dmin = 0xffffffffu;
-      s_dmax = 0u;
-      s_fmin = 0xffffffffu;
-    }
-    cluster_barrier();   // (also: every CTA runs before its shared memory is written)
+  if (ran && tid == 0) {
+    if (rank == 0) st->small_n = 0;
+    s_n = 0;
+    s_nwide = 0;
+    s_ndefer = 0;
+    s_far_n = 0;
+    s_par = 0;
+    s_budget = 0;
+    s_over = 0;
+    s_wide_items = 0u;
+    s_tot = 0ull;
+    s_dmin = 0xffffffffu;
+    s_dmax = 0u;
+    s_fmin = 0xffffffffu;
   }
+  // Whether the loop runs or not: every CTA has read the level header (base,
+  // count, max_levels, the frontier above) before CTA 0 may write it at the
+  // end, so all take the same L0 and `ran`; and every CTA is running before its
+  // shared memory is written. (A CTA that read the header after that write took
+  // a level K later, whose count slot may hold a small old level.)
+  cluster_barrier();
   while (ran) {
     const int cur = (L - L0) & 1, nxt = cur ^ 1;
     // ---- the round's size and window, the same in every CTA

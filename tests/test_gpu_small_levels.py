@@ -85,6 +85,29 @@ def test_distances(ctx, name):
             assert st["error"] == 0 and st["timeouts"] == 0
 
 
+def _alternating(pairs):
+    """Levels of 3 and 60 vertices in turn: with a limit between the two, a while body of two levels
+    that starts at a wide one ends before the next wide one, just after a narrow one."""
+    g, src = _fan(80 * pairs, [3, 60] * pairs, 11)
+    g.w = gen.uniform_int(11, gen.S_WEIGHT, 0, g.m, 1, 255).astype(np.uint32)
+    return g, src
+
+
+@pytest.mark.parametrize("unroll", [2, 3, 5, 8, 11, 15])
+def test_levels_left_to_the_grids(ctx, unroll):
+    """The loop at a body's end that finds too large a frontier leaves it to the grids as it is,
+    whatever the number of levels in the body."""
+    g, src = _alternating(100)
+    big = GRAPHS["rmat-17001"]()
+    for g, src in ((g, src), (big, 0)):
+        dg = DevGraph(g)
+        ref = oracle.sssp(g.row_ptr, g.col, g.w, src)
+        for kw in ({"small_parents": 1}, {"small_parents": 40, "sweep_parents": 0}, {}):
+            d, st = sssp(ctx, dg, src, npb.config("tca", unroll=unroll, **kw), stats=True)
+            np.testing.assert_array_equal(d, ref)
+            assert st["error"] == 0 and st["timeouts"] == 0
+
+
 def test_several_sources_share_the_window(ctx):
     """Queries of one call share one window, whatever their distances."""
     g = _road(150, 140, 1, 255)
