@@ -140,6 +140,7 @@ __global__ void __launch_bounds__(1024) level_small(Args a, cudaGraphConditional
   const int L0 = __ldcg(&st->base) + K;
   int L = L0;
   unsigned long long n_par = 0, n_items = 0, n_serial = 0;
+  __syncthreads();   // every warp has read the base before thread 0 may move it on (below, without a level run)
   // The level's frontier: from global memory at the first level; after a level
   // of this loop whose appends all fit the stage, from the stage itself (the
   // level's count in `staged`, -1 otherwise), so the next level starts without

@@ -173,3 +173,17 @@ def test_bfs_road(ctx, rows, cols):
     dg = DevGraph(g)
     for src in (0, g.n // 2):
         np.testing.assert_array_equal(bfs(ctx, dg, src, npb.config("tca")), oracle.bfs(g.row_ptr, g.col, src))
+
+
+@pytest.mark.parametrize("unroll", [1, 2, 3, 5, 8, 11, 15])
+def test_bfs_levels_left_to_the_grids(ctx, unroll):
+    """As test_levels_left_to_the_grids, for the one-CTA loop at the end of a body."""
+    g, src = _alternating(100)
+    big = GRAPHS["rmat-17001"]()
+    for g, src in ((g, src), (big, 0)):
+        dg = DevGraph(g)
+        ref = oracle.bfs(g.row_ptr, g.col, src)
+        for kw in ({"small_parents": 8}, {"small_parents": 40, "sweep_parents": 0}, {}):
+            lv, st = bfs(ctx, dg, src, npb.config("tca", unroll=unroll, **kw), stats=True)
+            np.testing.assert_array_equal(lv, ref)
+            assert st["error"] == 0 and st["levels"] == ref.max() + 1
