@@ -431,7 +431,9 @@ np_status plan_map(const BodyKernels& K, const np_config& cfg, int n, Plan* p) {
   // 16 KB, 6 of 8 at 32 KB, 3 of 16 at 64 KB, then one or two of 32
   p->child_threads = 128;
   while (p->child_threads < 1024 && p->child_smem > (size_t)p->child_threads * 128) p->child_threads *= 2;
-  NP_CK(cudaFuncSetAttribute(p->child, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p->child_smem));
+  // (the attribute belongs to the function on the device, which other contexts
+  // launch too: always the most any graph takes, never this graph's size)
+  NP_CK(cudaFuncSetAttribute(p->child, cudaFuncAttributeMaxDynamicSharedMemorySize, K.map_vertices / 8));
   return NP_OK;
 }
 

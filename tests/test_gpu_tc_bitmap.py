@@ -1,6 +1,8 @@
 """Triangle counting's child grid with adjacency bitmaps: list lengths around the 32- and
 128-entry runs, records longer than a chunk of edges, every CTA size its bitmap takes, and the
 change to the intersection per thread above the largest bitmap. Counts are exact."""
+import threading
+
 import numpy as np
 import pytest
 import torch
@@ -61,3 +63,44 @@ def test_bitmap_sizes(ctx, n):
     for v in mids[::3]:
         lists[int(v)] = np.sort(rng.choice(ids, int(rng.integers(1, min(150, len(ids)))), replace=False))
     assert _count(ctx, n, lists, child_block=32, cfactor=1) == _expected(lists)
+
+
+def test_two_contexts_in_two_threads():
+    """Bitmaps of 16 KB and 200 KB counted at the same time through contexts of their own: neither
+    call changes what the other's launch may take."""
+    jobs = []
+    for n in (131072, 1638400):
+        rng = np.random.default_rng(n)
+        ids = np.unique(rng.integers(n // 4, n, 900))
+        lists = {0: np.concatenate([np.arange(1, 300), ids[-200:]])}
+        for v in range(1, 300, 3):
+            lists[v] = np.sort(rng.choice(ids, int(rng.integers(40, 150)), replace=False))
+        deg = np.zeros(n + 1, np.int64)
+        for u, l in lists.items():
+            deg[u + 1] = len(l)
+        row_ptr = torch.from_numpy(np.cumsum(deg).astype(np.int32)).cuda()
+        col = torch.from_numpy(np.concatenate([np.asarray(lists[u], np.int32) for u in sorted(lists)])).cuda()
+        jobs.append((npb.make_csr(row_ptr, col), _expected(lists), row_ptr, col))
+    torch.cuda.synchronize()
+    start, errors = threading.Barrier(len(jobs)), []
+
+    def work(csr, want):
+        try:
+            with npb.Context(0) as c:
+                s = torch.cuda.Stream()
+                out = torch.zeros(400, dtype=torch.int64, device="cuda:0")
+                torch.cuda.synchronize()
+                start.wait(timeout=60)
+                for i in range(len(out)):
+                    npb.np_triangles(c.handle, csr, out[i:], npb.config("tca", threshold=1), stream=s)
+                s.synchronize()
+                assert (out == want).all()
+        except Exception as e:   # (reported by the main thread)
+            errors.append(e)
+
+    threads = [threading.Thread(target=work, args=j[:2]) for j in jobs]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
