@@ -379,7 +379,9 @@ np_status np_server_finished(np_server *s, int64_t *tickets, int32_t max, int32_
  * curve-order exclusive scan of N (offsets[ncurves] = total). Child item j
  * writes points[offsets[c] + j] = B(j / (N - 1)) in FP32. If the total
  * exceeds `cap`, curves that do not fit are skipped and NP_ERR_CAPACITY is
- * reported; offsets are always complete. */
+ * reported; offsets are always complete. A total beyond INT32_MAX is treated so
+ * whatever `cap` is: curves that end beyond it are skipped, and offsets beyond
+ * it hold INT32_MAX. */
 np_status np_bezier(np_ctx *ctx, const float *ctrl, int32_t ncurves, int32_t *offsets,
                     float *points, int64_t cap, const np_config *cfg, void *stream,
                     np_stats *stats);

@@ -420,7 +420,7 @@ np_status np_bezier(np_ctx* c, const float* ctrl, int32_t ncurves, int32_t* offs
   a.b.ctrl = ctrl;
   a.b.points = reinterpret_cast<float2*>(points);
   a.offsets = offsets;
-  a.cap = cap;
+  a.cap = cap < INT32_MAX ? cap : INT32_MAX;   // (offsets are int32)
   st = fixed_pass(c, a, *cfg, bezier_kernels(), ncurves, (cudaStream_t)stream);
   if (st != NP_OK) return st;
   return finish(c->e, c->w, (cudaStream_t)stream, stats);
@@ -495,7 +495,7 @@ np_status np_run_nested(np_ctx* c, const np_parents* parents, int32_t count_kind
     a.b.ctrl = body->ctrl;
     a.b.points = reinterpret_cast<float2*>(body->points);
     a.offsets = body->offsets;
-    a.cap = body->cap;
+    a.cap = body->cap < INT32_MAX ? body->cap : INT32_MAX;   // (offsets are int32)
   }
   st = fixed_pass(c, a, *cfg, *K, parents->count, s);
   if (st != NP_OK) return st;

@@ -134,7 +134,7 @@ extern "C" np_status np_bezier_noalloc(const float* ctrl, int32_t ncurves, int32
   a.child_block = cfg->child_block;
   a.scan = cfg->scan;
   a.offsets = offsets;
-  a.cap = cap;
+  a.cap = cap < INT32_MAX ? cap : INT32_MAX;   // (offsets are int32)
   a.b.st = state;
   a.b.vmask = 0x7fffffff;
   a.b.ctrl = ctrl;

@@ -118,10 +118,11 @@ __global__ void NP_PARENT_BOUNDS parent_kernel(Args a) {
       __syncthreads();
       const unsigned tile_base = s_v4.a;
       __syncthreads();
-      base = (int)(tile_base + e0);
+      const unsigned at = sat_add(tile_base, e0);
+      base = offset_word(at);
       if (valid) a.offsets[i] = base;
-      if (tile == ntiles - 1 && tid == 0) a.offsets[count] = (int)(tile_base + t0);
-      if (valid && (long long)base + N > a.cap) {
+      if (tile == ntiles - 1 && tid == 0) a.offsets[count] = offset_word(sat_add(tile_base, t0));
+      if (valid && (long long)at + N > a.cap) {
         atomicOr(&st->error, kErrCapacity);
         N = 0;
       }
@@ -374,14 +375,15 @@ __device__ __forceinline__ void parent_warp_run(const Args& a, int L, int count,
         }
         const unsigned gtot = __shfl_sync(kFull, tin, 31);
         const V4 x = lookback(a.ob_flag, a.ob_agg, a.ob_incl, grp, 0, epoch, V4{gtot, 0u, 0u, 0u}, st);
-        if (lane < nw) s_off[lane] = x.a + tin - t;   // exclusive prefix of each warp's tile
-        if (lane == 0) s_off[32] = x.a + gtot;
+        if (lane < nw) s_off[lane] = sat_add(x.a, tin - t);   // exclusive prefix of each warp's tile
+        if (lane == 0) s_off[32] = sat_add(x.a, gtot);
       }
       __syncthreads();
-      base = (int)(s_off[wid] + (unsigned)(inc - N));
+      const unsigned at = sat_add(s_off[wid], (unsigned)(inc - N));
+      base = offset_word(at);
       if (valid) a.offsets[i] = base;
-      if ((grp + 1) * nw >= ntiles && threadIdx.x == 0) a.offsets[count] = (int)s_off[32];
-      if (valid && (long long)base + N > a.cap) {
+      if ((grp + 1) * nw >= ntiles && threadIdx.x == 0) a.offsets[count] = offset_word(s_off[32]);
+      if (valid && (long long)at + N > a.cap) {
         atomicOr(&st->error, kErrCapacity);
         N = 0;
       }
@@ -614,10 +616,11 @@ __global__ void __maxnreg__(Body::kCtaParentRegs) parent_cta(Args a) {
       __syncthreads();
       const unsigned tile_base = s_x.a;
       __syncthreads();
-      base = (int)(tile_base + e0);
+      const unsigned at = sat_add(tile_base, e0);
+      base = offset_word(at);
       if (valid) a.offsets[i] = base;
-      if (tile == ntiles - 1 && tid == 0) a.offsets[count] = (int)(tile_base + t0);
-      if (valid && (long long)base + N > a.cap) {
+      if (tile == ntiles - 1 && tid == 0) a.offsets[count] = offset_word(sat_add(tile_base, t0));
+      if (valid && (long long)at + N > a.cap) {
         atomicOr(&st->error, kErrCapacity);
         N = 0;
       }

@@ -40,7 +40,8 @@ constexpr int kPointTile = kPointBlock;   // N <= 4096: an offset in the tile ta
 
 // np_stats and the total from what the threads of one CTA counted.
 __device__ __forceinline__ void point_stats(const Args& a, unsigned items, unsigned serial, unsigned launched,
-                                            unsigned citems, unsigned cblocks, unsigned curves, unsigned total) {
+                                            unsigned citems, unsigned cblocks, unsigned curves,
+                                            unsigned long long total) {
   __shared__ unsigned s_sum[6];
   const int tid = (int)threadIdx.x;
   if (tid < 6) s_sum[tid] = 0u;
@@ -63,53 +64,59 @@ __device__ __forceinline__ void point_stats(const Args& a, unsigned items, unsig
     st->s[S_PARENTS] = s_sum[5];
     st->body_iters = 0;
     if ((long long)total > a.cap) st->error |= kErrCapacity;
-    a.offsets[a.count_fixed] = (int)total;
+    a.offsets[a.count_fixed] = (int)min(total, (unsigned long long)INT_MAX);
   }
 }
 
 // Statistics and the total from the tiles' sums, by one CTA of kPointTile
-// threads; with `scan` the tiles' exclusive prefixes go to a.lb_incl as words.
+// threads; with `scan` the tiles' exclusive prefixes go to a.lb_incl as words
+// (at most kPointTop, beyond INT_MAX: nothing fits there, and the offset in the
+// tile can be added without wrapping).
+constexpr unsigned kPointTop = 0xfff00000u;
 __device__ __forceinline__ void point_totals(const Args& a, int ntiles, bool scan) {
   __shared__ uint2 s_scan2[33];
   const int tid = (int)threadIdx.x, count = a.count_fixed;
   const int T = a.threshold < 1 ? 1 : a.threshold;
   const bool never = a.threshold == INT_MAX;
   const int per = ceil_div(ntiles, kPointTile), t0 = min(tid * per, ntiles), t1 = min(t0 + per, ntiles);
-  unsigned items = 0, serial = 0, launched = 0, citems = 0, cblocks = 0, curves = 0;   // (offsets are 32 bits)
+  // (the counters fit in 32 bits where all points fit; else they are taken again below)
+  unsigned items = 0, serial = 0, launched = 0, citems = 0, cblocks = 0, curves = 0;
+  unsigned long long mine = 0;   // points of this thread's tiles: below 2^15 tiles of at most 2^20
 #pragma unroll 1
   for (int t = t0; t < t1; t++) {
     const uint4 v = __ldcg(&a.lb_agg[t]), x = __ldcg(&a.ob_agg[t]);
-    items += v.x;
+    mine += v.x;
     serial += v.y;
     launched += v.z;
     citems += v.w;
     cblocks += x.x;
     curves += x.y;
   }
-  unsigned e0, e1, total, u1;
-  block_scan2(items, 0u, e0, e1, total, u1, s_scan2);
-  const unsigned* tile0 = nullptr;
+  items = (unsigned)mine;
+  // a 64-bit scan of sums below 2^36 as two counters: the low 24 bits and the rest
+  unsigned e0, e1, lo, hi;
+  block_scan2((unsigned)mine & 0xffffffu, (unsigned)(mine >> 24), e0, e1, lo, hi, s_scan2);
+  const unsigned long long first = ((unsigned long long)e1 << 24) + e0, total = ((unsigned long long)hi << 24) + lo;
   if (scan) {
     unsigned* prefix = reinterpret_cast<unsigned*>(a.lb_incl);
+    unsigned long long at = first;
     for (int t = t0; t < t1; t++) {
-      prefix[t] = e0;
-      e0 += __ldcg(&a.lb_agg[t]).x;
+      prefix[t] = (unsigned)min(at, (unsigned long long)kPointTop);
+      at += __ldcg(&a.lb_agg[t]).x;
     }
-    tile0 = prefix;
-    __syncthreads();
   }
   if ((long long)total > a.cap) {
     // curves that do not fit have no children: count those that do (thread by
     // thread over its tiles' curves)
-    if (scan) e0 = t0 < ntiles ? __ldcg(&tile0[t0]) : 0u;
     items = serial = launched = citems = cblocks = 0;
-  #pragma unroll 1
-  for (int t = t0; t < t1; t++) {
+    unsigned long long at = first;
+#pragma unroll 1
+    for (int t = t0; t < t1; t++) {
 #pragma unroll 1
       for (int i = t * kPointTile; i < min(count, (t + 1) * kPointTile); i++) {
         const unsigned w = (unsigned)__ldcg(&a.boff[i]);
         const int N = (w & 4095u) ? (int)(w & 4095u) + 1 : 0;
-        if (N == 0 || (long long)(e0 + (w >> 12)) + N > a.cap) continue;
+        if (N == 0 || (long long)(at + (w >> 12)) + N > a.cap) continue;
         items += (unsigned)N;
         if (!never && N >= T) {
           launched++;
@@ -119,7 +126,7 @@ __device__ __forceinline__ void point_totals(const Args& a, int ntiles, bool sca
           serial++;
         }
       }
-      e0 += __ldcg(&a.lb_agg[t]).x;
+      at += __ldcg(&a.lb_agg[t]).x;
     }
   }
   point_stats(a, items, serial, launched, citems, cblocks, curves, total);
@@ -172,7 +179,7 @@ __global__ void __launch_bounds__(kPointTile, 4) bezier_count(Args a) {
 //
 // Lane l holds curve `i` = its warp's curve l % kPointCurves: id `pid` (-1: none),
 // offset and number of points.
-__device__ __forceinline__ void point_curves(const Args& a, int i, int pid, int base, int N) {
+__device__ __forceinline__ void point_curves(const Args& a, int i, int pid, unsigned base, int N) {
   const int lane = (int)threadIdx.x & 31;
   float ax = 0.f, ay = 0.f, bx = 0.f, by = 0.f, cx = 0.f, cy = 0.f;
   if (pid >= 0) {
@@ -184,7 +191,7 @@ __device__ __forceinline__ void point_curves(const Args& a, int i, int pid, int 
     by = __ldg(c + 3) * r2;
     cx = __ldg(c + 4) * r;
     cy = __ldg(c + 5) * r;
-    if (lane < kPointCurves) a.offsets[i] = base;
+    if (lane < kPointCurves) a.offsets[i] = offset_word(base);
   }
   if (pid < 0 || (long long)base + N > a.cap) N = 0;   // (none, or it does not fit: skipped)
   for (int q = 0; q < kPointCurves; q++) {
@@ -229,11 +236,12 @@ __global__ void __launch_bounds__(256, 6) bezier_points(Args a) {
   }
   const int first = ((int)blockIdx.x * ((int)blockDim.x >> 5) + ((int)threadIdx.x >> 5)) * kPointCurves;
   const int i = first + (lane & (kPointCurves - 1));
-  int base = 0, N = 0, pid = -1;
+  unsigned base = 0;
+  int N = 0, pid = -1;
   if (i < count) {
     const unsigned w = (unsigned)__ldcg(&a.boff[i]);
     pid = a.ids ? __ldcg(&a.ids[i]) : i;
-    base = (int)(before + (w >> 12));
+    base = before + (w >> 12);   // (at most 2^31 or so, or kPointTop and a tile: no wrap)
     N = (int)(w & 4095u) + 1;
   }
   point_curves(a, i, pid, base, N);
@@ -323,7 +331,7 @@ __global__ void __launch_bounds__(kPointBlock, 4) bezier_fused(Args a) {
   unsigned base = (unsigned)(incl - N);
 #pragma unroll
   for (int k = 0; k < kPointBlock / 32; k++) base += s_before[k] + (k < wid ? s_own[k] : 0u);
-  point_curves(a, i, pid, (int)base, N);
+  point_curves(a, i, pid, base, N);
 }
 
 }  // namespace nestpar

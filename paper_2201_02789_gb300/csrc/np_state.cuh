@@ -206,7 +206,7 @@ struct Args {
   const int* row_ptr;
   BodyArgs b;
   int* offsets;
-  long long cap;
+  long long cap;                 // tessellation: points that fit, at most INT_MAX
   int4* rec;
   int* boff;
   unsigned long long* lb_flag;   // look-back tile states of the aggregation scan
@@ -293,11 +293,21 @@ __device__ __forceinline__ unsigned pair_lo(unsigned long long w) { return (unsi
 struct V4 {
   unsigned a, b, c, d;
 };
-__device__ __forceinline__ V4 v4add(V4 x, V4 y) { return V4{x.a + y.a, x.b + y.b, x.c + y.c, x.d + y.d}; }
+// Point counts of all curves may pass 32 bits, offsets of points that fit never
+// do (Args::cap is at most INT_MAX): sums of them stay at the top instead of
+// wrapping, where nothing fits any more, and what is stored as an offset is at
+// most INT_MAX.
+__device__ __forceinline__ unsigned sat_add(unsigned a, unsigned b) {
+  const unsigned s = a + b;
+  return s < a ? 0xffffffffu : s;
+}
+__device__ __forceinline__ int offset_word(unsigned at) { return (int)min(at, (unsigned)INT_MAX); }
+// (the first counter is the one that carries output offsets)
+__device__ __forceinline__ V4 v4add(V4 x, V4 y) { return V4{sat_add(x.a, y.a), x.b + y.b, x.c + y.c, x.d + y.d}; }
 __device__ __forceinline__ V4 warp_sum4(V4 v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
-    v.a += __shfl_xor_sync(kFull, v.a, o);
+    v.a = sat_add(v.a, __shfl_xor_sync(kFull, v.a, o));
     v.b += __shfl_xor_sync(kFull, v.b, o);
     v.c += __shfl_xor_sync(kFull, v.c, o);
     v.d += __shfl_xor_sync(kFull, v.d, o);

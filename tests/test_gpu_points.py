@@ -65,6 +65,52 @@ def test_capacity_inside_a_tile(ctx, nc):
     assert st["items"] == ref_off[inside]
 
 
+WIDE_FORMS = {
+    "points": {}, "count-grid-3": dict(threshold=npb.INT32_MAX, parent_grid=3), "nodp": dict(variant=npb.NP_VARIANT_NODP),
+    "nodp-cta": dict(variant=npb.NP_VARIANT_NODP, granularity="none"), "cta": dict(serial=npb.NP_SERIAL_BLOCK),
+    "packed": dict(serial=npb.NP_SERIAL_PACKED), "none": dict(granularity="none"), "warp": dict(granularity="warp"),
+    "block": dict(granularity="block"), "grid_device": dict(granularity="grid_device", scan=npb.NP_SCAN_LOOKBACK),
+}
+
+
+def _closed(n):
+    """n curves that end where they begin: 4096 points each."""
+    ctrl = np.zeros((n, 3, 2), np.float32)
+    ctrl[:, 1] = [0.5, 0.25]
+    return torch.from_numpy(ctrl).cuda()
+
+
+@pytest.mark.parametrize("nc", [(1 << 19) + 77, (1 << 20) + 300], ids=["above-2^31", "above-2^32"])
+@pytest.mark.parametrize("form", list(WIDE_FORMS))
+def test_totals_beyond_32_bits(ctx, form, nc):
+    """More points than an int32 offset can number: the curves that end within the capacity are
+    written and nothing else, offsets beyond INT32_MAX hold INT32_MAX."""
+    c_d, cap, guard = _closed(nc), 10000, 1 << 22
+    off = torch.full((nc + 1,), -7, dtype=torch.int32, device="cuda:0")
+    pts = torch.full((guard + cap + guard, 2), float("nan"), dtype=torch.float32, device="cuda:0")
+    status, st = npb.np_bezier(ctx.handle, c_d, nc, off, pts[guard:], cap, npb.config("tca", **WIDE_FORMS[form]),
+                               stats=True, check=False)
+    assert status == npb.NP_ERR_CAPACITY
+    want = np.minimum(np.arange(nc + 1, dtype=np.int64) * 4096, npb.INT32_MAX)
+    np.testing.assert_array_equal(off.cpu().numpy(), want)
+    written = ~torch.isnan(pts[:, 0])
+    assert written[guard:guard + 8192].all() and int(written.sum()) == 8192
+    assert st["items"] == 8192 and st["parents"] == nc
+
+
+def test_capacity_beyond_32_bits(ctx):
+    """A buffer of more than 2^31 points: what ends beyond INT32_MAX is skipped all the same."""
+    nc = (1 << 19) + 2
+    c_d, cap = _closed(nc), nc * 4096
+    off = torch.full((nc + 1,), -7, dtype=torch.int32, device="cuda:0")
+    pts = torch.full((cap, 2), float("nan"), dtype=torch.float32, device="cuda:0")
+    status, st = npb.np_bezier(ctx.handle, c_d, nc, off, pts, cap, npb.config("tca"), stats=True, check=False)
+    assert status == npb.NP_ERR_CAPACITY
+    fit = (npb.INT32_MAX // 4096) * 4096
+    assert torch.isfinite(pts[fit - 4096:fit]).all() and torch.isnan(pts[fit:]).all()
+    assert st["items"] == fit
+
+
 def test_parent_subset_with_padding(ctx):
     ctrl = gen.bezier_curves(600, seed=53)
     ids = np.arange(599, -1, -1, dtype=np.int32)[:520].copy()
