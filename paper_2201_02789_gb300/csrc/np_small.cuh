@@ -118,9 +118,13 @@ __device__ __forceinline__ int warp_segment(const int4* seg, int n, int t) {
 //
 // An entry of a far list carries the distance its vertex had when it was
 // deferred; if the vertex has been lowered since, that lowering pushed an
-// entry of its own and the old one is dropped. So a vertex has at most one
+// entry of its own and the old one is dropped. Nothing separates the CTAs'
+// pulls of a round from their relaxations, so a pulled vertex may already have
+// been lowered in the same round: its tag is then the round's own, and the
+// pulled entry is dropped too, because that lowering pushed one (deferred with
+// the new distance as its key, both would be live). So a vertex has at most one
 // live entry, and when the grids take over (a frontier too large) the live
-// entries are the frontier. Windowed rounds are not Bellman-Ford levels: the
+// entries are the frontier, no more than there are vertices. Windowed rounds are not Bellman-Ford levels: the
 // level cap moves on by the rounds run here, and a run of the loop is bounded
 // by its own count of rounds.
 constexpr int kSmallParentsMax = 2048;
@@ -304,10 +308,13 @@ __global__ void __launch_bounds__(kClThreads) sssp_cluster(Args a, cudaGraphCond
 #pragma unroll
     for (int r = 0; r < kClPull + kClFar; r++) {
       use[r] = pid[r] >= 0 && (r < kClPull || key[r < kClPull ? 0 : r - kClPull] <= cut);
-      d[r] = use[r] ? (unsigned)(__ldcg(&a.b.dtag[pid[r]]) >> 32) : 0u;
+      const unsigned long long word = use[r] ? __ldcg(&a.b.dtag[pid[r]]) : 0ull;
+      d[r] = (unsigned)(word >> 32);
       base[r] = 0;
       N[r] = 0;
       if (use[r]) Body::count(a, pid[r], base[r], N[r]);
+      // (lowered in this round: an entry of the next one)
+      if (r < kClPull) use[r] = use[r] && (unsigned)word != (unsigned)(L + 1);
     }
 #pragma unroll
     for (int r = 0; r < kClWide; r++) {
