@@ -24,7 +24,7 @@ namespace nestpar {
 // tiles waited for its look-back before it could store its first point, and a
 // CTA held 450-500 curves, too coarse to fill 152 SMs. Measured, one pass of
 // random curves (6.2 M and 25 M points, threshold 32 and none): 43.9 -> 15.1 us
-// and 64.8 -> 42.6 us; the point grid alone takes 34 us for 25 M points (200 MB
+// and 64.8 -> 43.2 us; the point grid alone takes 35 us for 25 M points (200 MB
 // of stores, 30 us at the copy bandwidth; 68% of the issue slots).
 static_assert(kPointBlock % (kPointBlock / 32 * kPointCurves) == 0, "a point CTA's curves lie in one count tile");
 constexpr int kPointTile = kPointBlock;   // N <= 4096: an offset in the tile takes 20 bits
@@ -177,24 +177,40 @@ __global__ void __launch_bounds__(kPointTile, 4) bezier_count(Args a) {
 // then runs them one after the other from shuffles: 17 instructions per 32
 // points and 14 per curve.
 //
+// The products keep their 24 bits only while they are normal numbers (r is at
+// least 2^-24): a curve with a coordinate below 2^-100 in magnitude, other than
+// 0, takes the child body's own form instead, whose weights carry r and whose
+// coordinates are not scaled. (Scaled all the same, coordinates of 1e-36 came
+// out with a relative error of 1.2e-2 at N = 4096; the test takes 1 us of the
+// point grid's 35 for 25 M points, weights that carry r in every curve 2.8.)
+//
 // Lane l holds curve `i` = its warp's curve l % kPointCurves: id `pid` (-1: none),
 // offset and number of points.
 __device__ __forceinline__ void point_curves(const Args& a, int i, int pid, unsigned base, int N) {
   const int lane = (int)threadIdx.x & 31;
   float ax = 0.f, ay = 0.f, bx = 0.f, by = 0.f, cx = 0.f, cy = 0.f;
+  bool low = false;
   if (pid >= 0) {
     const float* c = a.b.ctrl + 6 * (size_t)pid;
     const float nm1 = (float)(N - 1), r = 1.0f / (nm1 * nm1), r2 = 2.0f * r;
-    ax = __ldg(c) * r;
-    ay = __ldg(c + 1) * r;
-    bx = __ldg(c + 2) * r2;
-    by = __ldg(c + 3) * r2;
-    cx = __ldg(c + 4) * r;
-    cy = __ldg(c + 5) * r;
+    ax = __ldg(c);
+    ay = __ldg(c + 1);
+    bx = __ldg(c + 2);
+    by = __ldg(c + 3);
+    cx = __ldg(c + 4);
+    cy = __ldg(c + 5);
+    low = fminf(fminf(fminf(fabsf(ax), fabsf(ay)), fminf(fabsf(bx), fabsf(by))), fminf(fabsf(cx), fabsf(cy))) < 0x1p-100f;
+    ax *= r;
+    ay *= r;
+    bx *= r2;
+    by *= r2;
+    cx *= r;
+    cy *= r;
     if (lane < kPointCurves) a.offsets[i] = offset_word(base);
   }
-  if (pid < 0 || (long long)base + N > a.cap) N = 0;   // (none, or it does not fit: skipped)
-  for (int q = 0; q < kPointCurves; q++) {
+  // (none, or it does not fit: skipped; the capacity is at most INT_MAX)
+  if (pid < 0 || offset_word(base) > (int)a.cap - N) N = 0;
+  auto scaled = [&](int q) {
     const int n = __shfl_sync(kFull, N, q);
     float2* out = a.b.points + __shfl_sync(kFull, base, q) + lane;
     const float x0 = __shfl_sync(kFull, ax, q), y0 = __shfl_sync(kFull, ay, q), x1 = __shfl_sync(kFull, bx, q),
@@ -206,6 +222,36 @@ __device__ __forceinline__ void point_curves(const Args& a, int i, int pid, unsi
       out += 32;
       j += 32.0f;
       k -= 32.0f;
+    }
+  };
+  if (!__any_sync(kFull, low)) {
+    for (int q = 0; q < kPointCurves; q++) scaled(q);
+    return;
+  }
+  // (a zero stays a zero: no reason by itself)
+  bool tiny = false;
+  if (low)
+    for (int k = 0; k < 6; k++) {
+      const float x = fabsf(__ldg(a.b.ctrl + 6 * (size_t)pid + k));
+      tiny = tiny || (x > 0.0f && x < 0x1p-100f);
+    }
+  const unsigned apart = __ballot_sync(kFull, tiny);
+#pragma unroll 1
+  for (int q = 0; q < kPointCurves; q++) {
+    if (!(apart >> q & 1u)) {   // (uniform)
+      scaled(q);
+      continue;
+    }
+    const int n = __shfl_sync(kFull, N, q);
+    const BezierBody::P p[1] = {
+        BezierBody::parent(a.b, __shfl_sync(kFull, pid, q), (int)__shfl_sync(kFull, base, q), n)};
+    for (int j = lane; j < n; j += 32) {
+      const int idx[1] = {j};
+      const BezierBody::F f[1] = {};
+      const bool v[1] = {true};
+      bool push[1];
+      int next[1];
+      BezierBody::apply_batch<1>(a.b, p, idx, f, v, push, next);
     }
   }
 }

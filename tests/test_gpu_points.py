@@ -198,3 +198,39 @@ def test_after_device_launched_children(ctx, gran):
         npb.np_bezier(ctx.handle, a, 3000, off, pts, 600000, npb.config("tca", granularity=gran, threshold=0))
         npb.np_bezier(ctx.handle, b, 300, off, pts, 600000)
         assert int(off[300].item()) == total and torch.equal(pts[:total], ref)
+
+
+def _scaled_curves(n, seed):
+    """Curves of all magnitudes down to the smallest subnormal: whole curves scaled, x and y scaled
+    apart, single coordinates; every fourth one closed (4096 points)."""
+    rng = np.random.default_rng(seed)
+    u = rng.uniform(-1, 1, (n, 3, 2))
+    e = rng.integers(-149, 3, (n, 1, 1)).astype(np.float64)
+    e = np.where(np.arange(n)[:, None, None] % 3 == 1, rng.integers(-149, 3, (n, 1, 2)), e)
+    e = np.where(np.arange(n)[:, None, None] % 3 == 2, rng.integers(-149, 3, (n, 3, 2)), e)
+    ctrl = (u * 2.0 ** e).astype(np.float32)
+    ctrl[::4, 2] = ctrl[::4, 0]
+    return np.ascontiguousarray(ctrl)
+
+
+@pytest.mark.parametrize("nc", [300, 3000])
+@pytest.mark.parametrize("kw", [{}, {"threshold": npb.INT32_MAX, "parent_grid": 3}])
+def test_points_of_any_magnitude(ctx, nc, kw):
+    """Each coordinate to 9 units of 2^-24 of the sum of its three terms' magnitudes and 4 halves
+    of the smallest subnormal. The longest chain: the reciprocal, t and u by it (two roundings each,
+    in a product of two of them), that product, its product with the coordinate and two sums: 8; one
+    more for second-order terms. A rounding to a subnormal is half of 2^-149, three products and
+    the sums at most four of them."""
+    ctrl = _scaled_curves(nc, seed=56)
+    ref_off = oracle.bezier_offsets(ctrl)
+    status, off, pts, _ = bezier(ctx, ctrl, npb.config("tca", **kw), cap=int(ref_off[-1]))
+    assert status == npb.NP_OK
+    np.testing.assert_array_equal(off, ref_off)
+    n_of = np.diff(ref_off)
+    curve = np.repeat(np.arange(nc), n_of)
+    j = (np.arange(ref_off[-1]) - ref_off[:-1][curve]).astype(np.float64)
+    t, u = j / (n_of[curve] - 1), (n_of[curve] - 1 - j) / (n_of[curve] - 1)
+    terms = np.stack([u * u, 2 * u * t, t * t], 1)[:, :, None] * ctrl.astype(np.float64)[curve]
+    bound = 9 * 2.0 ** -24 * np.abs(terms).sum(1) + 4 * 2.0 ** -150
+    worst = (np.abs(pts.astype(np.float64) - terms.sum(1)) / bound).max()
+    assert worst <= 1.0, worst
