@@ -32,6 +32,18 @@ __device__ __forceinline__ void st_release_u32(unsigned* p, unsigned v) {
   asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
+// A CTA barrier that counts threads, whichever way they arrive; __syncthreads
+// (an aligned bar.sync) counts whole warps and relies on each being together.
+// At the barrier after thread 0's part below that did not hold in a build of
+// level_loop with more spilled registers: the other warps got past it before
+// thread 0 had arrived, read *s_ok and, in later levels, the frontier's count
+// before they were written, and left the loop. (A __syncwarp before it, a wait
+// by the whole warp, fences and volatile reads changed nothing, nor did this
+// form at the first barrier, which there costs 8%; here it costs nothing.)
+__device__ __forceinline__ void cta_barrier_by_thread() {
+  asm volatile("barrier.sync 0;" ::: "memory");
+}
+
 // Returns false (in every thread of the CTA) once any CTA has timed out.
 __device__ __forceinline__ bool grid_barrier(LevelState* st, int* s_ok, unsigned long long limit_ns = kBarrierNs) {
   __syncthreads();
@@ -59,10 +71,16 @@ __device__ __forceinline__ bool grid_barrier(LevelState* st, int* s_ok, unsigned
     }
     *s_ok = ok && !(__ldcg(&st->error) & kErrTimeout);
   }
-  __syncthreads();
+  cta_barrier_by_thread();
   return *s_ok != 0;
 }
 
+// Parent tiles by the fixed stride with loads ahead, as in the parent grid
+// (parent_warp_run)? Both phases of the loop share 64 registers, and the loads
+// ahead spill 10 of them or more: by default the tiles come from the ticket.
+#ifndef NP_LOOP_AHEAD
+#define NP_LOOP_AHEAD 0
+#endif
 template <class Body, int FORM, int CF>
 __global__ void __launch_bounds__(1024) level_loop(Args a, int max_levels) {
   __shared__ int s_stage[kCtaStage];
@@ -73,7 +91,7 @@ __global__ void __launch_bounds__(1024) level_loop(Args a, int max_levels) {
     const int count = __ldcg(&st->count[L % 3]);
     if (count <= 0) break;   // uniform: every CTA reads it after the same barrier
     if (blockIdx.x == 0 && threadIdx.x == 0) level_open(st, L, count);
-    parent_warp_run<Body, FORM, 0>(a, L, count, false, s_stage, &s_stage_n, &s_stage_base);
+    parent_warp_run<Body, FORM, NP_LOOP_AHEAD>(a, L, count, false, s_stage, &s_stage_n, &s_stage_base);
     if constexpr (FORM == 1) {
       if (!grid_barrier(st, &s_ok)) break;
       BodyArgs b = a.b;

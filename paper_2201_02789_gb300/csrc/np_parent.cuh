@@ -255,8 +255,7 @@ __global__ void NP_PARENT_BOUNDS parent_kernel(Args a) {
 // loop (lanes with fewer children idle) that appends through a warp sink. No
 // CTA barrier anywhere, so no warp waits for another warp's serial loop.
 constexpr int kStaticT = 128;
-// AHEAD 0: later tiles always from the ticket (the persistent loop, whose
-// registers are taken by both phases).
+// AHEAD 0: later tiles always from the ticket (the persistent loop, see NP_LOOP_AHEAD).
 template <class Body, int FORM, int AHEAD = 1>
 __device__ __forceinline__ void parent_warp_run(const Args& a, int L, int count, bool fixed, int* s_stage,
                                                 int* s_stage_n, int* s_stage_base) {
