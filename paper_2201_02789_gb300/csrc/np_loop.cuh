@@ -147,7 +147,6 @@ __global__ void __launch_bounds__(1024) level_small(Args a, cudaGraphConditional
   __shared__ int s_first[PPT * 1024];
   __shared__ int s_pid[PPT * 1024];
   __shared__ int s_base[PPT * 1024];
-  __shared__ unsigned s_aux[PPT * 1024];
   __shared__ uint2 s_scan[33];
   __shared__ int s_stage[kCtaStage];
   __shared__ int s_stage_n, s_stage_base;
@@ -171,7 +170,6 @@ __global__ void __launch_bounds__(1024) level_small(Args a, cudaGraphConditional
     if (count <= 0 || count > limit || L >= max_levels) break;
     const int* ids = staged >= 0 ? s_stage : ((L & 1) ? a.fr1 : a.fr0);
     int pid[PPT], base[PPT], N[PPT];
-    unsigned aux[PPT];
     bool valid[PPT];
     unsigned mine = 0;
     BodyArgs b = a.b;
@@ -185,8 +183,6 @@ __global__ void __launch_bounds__(1024) level_small(Args a, cudaGraphConditional
       base[r] = 0;
       N[r] = 0;
       if (valid[r]) Body::count(a, pid[r], base[r], N[r]);
-      // (the value a staged parent carries, loaded beside its row bounds)
-      aux[r] = valid[r] ? Body::aux(b, pid[r]) : 0u;
       mine += (unsigned)N[r];
     }
     unsigned e0, e1, items, t1;
@@ -209,7 +205,6 @@ __global__ void __launch_bounds__(1024) level_small(Args a, cudaGraphConditional
           s_first[i] = (int)first;
           s_pid[i] = pid[r];
           s_base[i] = base[r];
-          s_aux[i] = aux[r];
         }
         first += (unsigned)N[r];
       }
@@ -231,8 +226,8 @@ __global__ void __launch_bounds__(1024) level_small(Args a, cudaGraphConditional
         for (int step = top; step > 0; step >>= 1)
           if (r + step < count && s_first[r + step] <= t) r += step;
         idx[k] = t - s_first[r];
-        // (the level-loop bodies do not use N in parent_aux)
-        pk[k] = Body::parent_aux(b, s_pid[r], s_base[r], 0, s_aux[r]);
+        // (BFS uses neither N nor a staged value of its parents)
+        pk[k] = Body::parent_aux(b, s_pid[r], s_base[r], 0, 0u);
         f[k] = v[k] ? Body::fetch(b, pk[k], idx[k]) : typename Body::F{};
       }
       bool pf[KS];
