@@ -869,13 +869,12 @@ def run_ours(args, ws, rank, local):
             "vs_baseline": None, "dtype": {"bezier": "f32", "tc": "i32"}.get(wl["kind"], "u32"), "data": "synthetic",
             "config": dict(wl["config"], l2=L2_NOTE),
             "form": (("threshold INT32_MAX (no child launches: a count grid over the curves, then a grid over "
-                      "their points, one warp per curve), " if wl["kind"] == "bezier" else
+                      "their points, a warp per eight curves), " if wl["kind"] == "bezier" else
                       "threshold INT32_MAX (no child launches: the serialised children spread over the "
                       "parent warps), ") if cfg.threshold == npb.INT32_MAX else
                      f"threshold {cfg.threshold} + coarsening {cfg.cfactor} ({cfg.child_block}-thread child blocks) "
                      "+ grid aggregation (atomic scan), ") + (
-                        "one fixed pass" if wl["kind"] == "bezier" else
-                        "one fixed pass replayed as a CUDA graph" if wl["kind"] == "tc" else
+                        "one fixed pass" if wl["kind"] in ("bezier", "tc") else
                         f"persistent cooperative level loop on {cfg.parent_grid} CTAs"
                         if cfg.driver == npb.NP_DRIVER_PERSISTENT else "while-graph level loop"),
             "ms_per_solve": {"median": statistics.median(ms), "min": min(ms)},

@@ -178,14 +178,24 @@ typedef struct np_csr {       /* CSR digraph, device pointers */
   int64_t m;                  /* edges, 0 <= m < 2^31 */
 } np_csr;
 
-typedef struct np_stats {     /* device-side counters of the last call */
-  uint64_t levels;            /* non-empty levels / iterations run */
+/* Device-side counters of the last call. Two forms count in their own way:
+ *   - an SSSP solve that runs rounds in the small-level cluster (`small_parents`,
+ *     on by default): a round may leave the farther part of a frontier to later
+ *     rounds, so `levels` is the number of rounds, not the Bellman-Ford depth, and
+ *     `parents`, `items` and `pushes` count what the rounds ran;
+ *   - the tessellation under grid-host aggregation with spread children: one grid
+ *     runs the points of all curves, whatever the threshold. `serial_parents`,
+ *     `launch_parents`, `child_items` and `child_blocks` are what the form defines
+ *     for the configuration (which curves reach the threshold, their points and
+ *     coarsened blocks), not grids or blocks that ran. */
+typedef struct np_stats {
+  uint64_t levels;            /* non-empty levels / iterations / rounds run */
   uint64_t parents;           /* parent threads that ran (frontier pops) */
   uint64_t serial_parents;    /* parents with N > 0 that serialised their children */
   uint64_t launch_parents;    /* parents whose children ran in a child grid */
   uint64_t device_launches;   /* device-side kernel launches performed */
   uint64_t aggregated_grids;  /* of which aggregated child grids */
-  uint64_t child_blocks;      /* coarsened child blocks executed */
+  uint64_t child_blocks;      /* coarsened child blocks executed (tessellation: see above) */
   uint64_t items;             /* child items executed (edges visited/relaxed, points) */
   uint64_t pushes;            /* vertices appended to frontiers */
   uint64_t launch_failures;   /* refused device launches (serialised instead) */

@@ -254,6 +254,16 @@ __global__ void NP_PARENT_BOUNDS parent_kernel(Args a) {
 // slots and block offsets, and the serialised children run in a warp-uniform
 // loop (lanes with fewer children idle) that appends through a warp sink. No
 // CTA barrier anywhere, so no warp waits for another warp's serial loop.
+//
+// The largest threshold whose tiles go by the fixed stride (below). Microseconds
+// a solve, ticket / fixed stride, at thresholds 64, 128, 256, 512:
+//   SSSP R-MAT 2^20            438 / 427    455 / 469    555 / 620    553 / 620
+//   BFS R-MAT 2^20             172 / 168    174 / 177    203 / 215    203 / 215
+//   16 SSSP sources, 2^18     1316 / 1222  1325 / 1325  1327 / 1329  1465 / 1690
+//   SSSP Zipf(2.1) 2^20        756 / 578    744 / 571    753 / 575    764 / 595
+// Up to 128 the fixed stride wins 23% or loses 3%; above it loses 10% and more
+// where serialised children differ widely (R-MAT), though not on a Zipf graph,
+// whose degrees are small.
 constexpr int kStaticT = 128;
 // AHEAD 0: later tiles always from the ticket (the persistent loop, see NP_LOOP_AHEAD).
 template <class Body, int FORM, int AHEAD = 1>
